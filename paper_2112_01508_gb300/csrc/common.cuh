@@ -13,7 +13,8 @@ constexpr int kWarp = 32;
 constexpr int kMaxDrifts = 64;  // drifts of the sorted positions allowed between two sorts
 constexpr int kChunk = 32;  // receivers per chunk (one warp lane each)
 constexpr int kPartItems = 32768;  // work items of split chunks that the partial-sum buffer holds
-constexpr int kMaxParts = 8;       // parts a chunk is split into at most
+constexpr int kMaxParts = 8;       // parts a chunk is split into at most (FP32)
+constexpr int kPartItemsPerChunk = 48;  // items of the buffer per chunk of a small set (32 parts of three doubles)
 
 // Device-side error bits, latched in a device word by the kernels.
 enum : int {

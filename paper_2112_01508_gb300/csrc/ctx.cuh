@@ -36,7 +36,8 @@ struct p3m_sr_ctx {
   int* act_scan = nullptr;            // n + 1
   int* active_idx = nullptr;          // n
   int* tile_chunks = nullptr;         // n_tiles + 1 (chunks per row segment, scanned)
-  float4* part_acc = nullptr;         // partial sums of split chunks (work items x 32 lanes)
+  float4* part_acc = nullptr;         // partial sums of split chunks (part_items work items x 32 lanes)
+  int part_items = 0;
   p3m::Chunk* chunks = nullptr;       // receiver chunks of the last build_pairs
   p3m::Chunk* chunks_all = nullptr;   // chunks over all particles (vjp)
   int64_t max_chunks = 0;
@@ -52,6 +53,7 @@ struct p3m_sr_ctx {
   double* abar_d = nullptr;           // vjp: masked abar, FP64 (3 n)
   float* table = nullptr;             // tabulated bracket (p3m_sr_forces_tabulated)
   int table_bits = 0;
+  double* tab64 = nullptr;            // polynomials of the FP64 pair bracket (pair_tables.cuh)
 
   // ---- error latch ----
   int* err_dev = nullptr;
@@ -91,6 +93,12 @@ p3m_status poll_latched(p3m_sr_ctx* ctx);
 void report_latched(p3m_sr_ctx* ctx);
 // Build (if needed) the chunk list over all particles.
 p3m_status ensure_all_chunks(p3m_sr_ctx* ctx);
+// The FP64 kernels' tables (pair64.cu): their size, and filling ctx->tab64 on the stream.
+int64_t pair_table_doubles();
+p3m_status fill_pair_tables(p3m_sr_ctx* ctx);
+// FP64 forces or adjoint on the chunks of `a`.
+struct TraversalArgs;
+cudaError_t launch_pair64(p3m_sr_ctx* ctx, const TraversalArgs& a, bool vjp);
 
 }  // namespace p3m
 

@@ -36,14 +36,11 @@
 
 #include <type_traits>
 
-#include "ctx.cuh"
 #include "erfcx_fit.h"
-#include "pair_math.cuh"
+#include "traverse.cuh"
 
 namespace p3m {
 
-constexpr int kForceThreads = 128;
-constexpr int kForceWarps = kForceThreads / kWarp;
 // Supplier subtiles buffered per warp before their particles are walked: 256
 // measured best on the 128^3 and 512^3 sets (the one-sided kernel 4-8% faster than
 // with 128, the each-pair-once kernel unchanged; 64 slower).
@@ -267,343 +264,15 @@ __global__ void k_abar_f64(const double* __restrict__ abar, const int8_t* __rest
 }
 
 // ---------------------------------------------------------------------------
-// The traversal kernel.
+// FP32 kernels (the traversal they share with the FP64 ones is in traverse.cuh).
 // ---------------------------------------------------------------------------
 
-struct TraversalArgs {
-  Geometry g;
-  ForceConsts f;
-  SeriesConsts sc;
-  const double* pos;          // FP64 path positions
-  const float4* rel4;         // FP32 path coordinates
-  const int* offsets;         // S + 1 subtile offsets
-  const int* cell;            // sorted subtile ids
-  const Chunk* chunks;
-  float4* part_acc;           // per (work item, lane) partial sums when chunks are split (kPartItems x 32), or nullptr
-  const float* drift_slots;   // displacement bounds of the drifts since the sort (device)
-  int n_drift;                // how many of them
-  int* err;                   // device error bits (kErrDrift), or nullptr
-  const int* n_chunks;        // device count
-  int* counter;               // dynamic chunk counter (zeroed before launch)
-  const int* active_idx;      // receiver list (nullptr: chunk ranges are particle indices)
-  int64_t n;
-  void* out;                  // acc (forward) or xbar (vjp), 3 x n
-  // vjp only
-  const float4* abar4;        // masked abar FP32
-  const double* abar_d;       // masked abar FP64, 3 x n
-  unsigned long long* pairs;  // interacting ordered pairs
-  // tabulated bracket (p3m_sr_forces_tabulated): B at the centres of n_table
-  // equal bins of r^2 in [0, x_r^2)
-  const float* table;
-  int n_table;
-  float table_scale;          // n_table / x_r^2
-};
+using WarpList = WarpListOf<kListCap>;
 
-template <class Real>
-struct Vec3 {
-  Real x, y, z;
-};
-
-__device__ __forceinline__ float redux_min_f(float v) {
-  float r;
-  asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ float redux_max_f(float v) {
-  float r;
-  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ double warp_min_d(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double warp_max_d(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float warp_min(float v) { return redux_min_f(v); }
-__device__ __forceinline__ float warp_max(float v) { return redux_max_f(v); }
-__device__ __forceinline__ double warp_min(double v) { return warp_min_d(v); }
-__device__ __forceinline__ double warp_max(double v) { return warp_max_d(v); }
-
-__device__ __forceinline__ unsigned pack_delta(int dx, int dy, int dz) {
-  return ((unsigned)(dx + 512) << 20) | ((unsigned)(dy + 512) << 10) | (unsigned)(dz + 512);
-}
-__device__ __forceinline__ void unpack_delta(unsigned p, int& dx, int& dy, int& dz) {
-  dx = (int)(p >> 20) - 512;
-  dy = (int)((p >> 10) & 1023u) - 512;
-  dz = (int)(p & 1023u) - 512;
-}
-
-struct WarpList {
-  int start[kListCap];
-  int pre[kListCap];       // exclusive prefix of the supplier counts
-  unsigned delta[kListCap];
-};
-
-// Reach of the traversal.  Right after a sort: the block R of subtiles around the
-// receivers' subtiles and the pruning bound x_r on the gap between a candidate
-// subtile box and the receivers' box.  After drifts of total length delta since
-// the sort, a particle may lie up to delta outside the subtile it was sorted into:
-// the gap bound grows to x_r + delta and the block to x_r + 2 delta (receivers and
-// suppliers both moved).
-struct Reach {
-  int R[3];
-  float sub2;     // squared gap bound, FP32 path
-  double sub2_d;  // FP64 path
-};
-
-__device__ __forceinline__ Reach make_reach(const TraversalArgs& a) {
-  Reach r;
-  float delta = 0.0f;
-  for (int k = 0; k < a.n_drift; ++k) delta += a.drift_slots[k];
-  if (!(delta > 0.0f)) {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) r.R[d] = a.g.R[d];
-    r.sub2 = a.f.margin2_f;
-    r.sub2_d = (double)a.f.margin2_f;
-    return r;
-  }
-  const double dl = (double)delta * (1.0 + 1e-5);  // the float sum may round down
-  const double reach = sqrt((double)a.f.margin2_f) + dl;
-  if (!(reach + dl < 0.5 * a.g.box)) {
-    if ((threadIdx.x & 31) == 0 && a.err) atomicOr(a.err, kErrDrift);
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const double rr = fmin(reach + dl, 0.5 * a.g.box);
-    r.R[d] = (int)ceil(rr / a.g.side64[d] * (1.0 + 1e-12));
-  }
-  r.sub2_d = reach * reach;
-  r.sub2 = (float)(r.sub2_d * (1.0 + 1e-6));
-  return r;
-}
-
-// The receivers of one chunk in its frame: positions, bounding box, subtile block.
-template <class Real>
-struct ChunkFrame {
-  bool valid;       // this lane holds a receiver
-  int pidx;         // its sorted particle index
-  int g0[3];        // subtile of lane 0 (frame origin)
-  Vec3<Real> pi;    // receiver position (chunk frame in FP32, absolute in FP64)
-  Vec3<Real> lo, hi;  // bounding box of the receivers
-  int elo[3], ext[3];  // candidate subtile block (offsets from g0) and its extent
-  float inv_ext[2];    // 1 / ext[2], 1 / ext[1], for decoding candidate indices
-  Real org[3];      // position of g0's origin in the frame
-};
-
-template <class Real>
-__device__ __forceinline__ void load_chunk(const TraversalArgs& a, const Reach& rc, const Chunk& ch, int lane,
-                                           ChunkFrame<Real>& F) {
-  const unsigned full = 0xffffffffu;
-  const Geometry& g = a.g;
-  F.valid = lane < ch.count;
-  F.pidx = 0;
-  if (F.valid) F.pidx = a.active_idx ? a.active_idx[ch.start + lane] : ch.start + lane;
-  int gi[3] = {0, 0, 0};
-  float4 ri = make_float4(0.f, 0.f, 0.f, 0.f);
-  {
-    int id = 0;
-    if constexpr (sizeof(Real) == 4) {
-      if (F.valid) ri = a.rel4[F.pidx];
-      id = __float_as_int(ri.w);
-    } else {
-      if (F.valid) id = a.cell[F.pidx];
-    }
-    if (F.valid) decode_subtile(g, id, gi[0], gi[1], gi[2]);
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) F.g0[d] = __shfl_sync(full, gi[d], 0);
-  const int e[3] = {gi[0] - F.g0[0], gi[1] - F.g0[1], gi[2] - F.g0[2]};
-  if constexpr (sizeof(Real) == 4) {
-    F.pi.x = fmaf((float)e[0], g.side32[0], ri.x);
-    F.pi.y = fmaf((float)e[1], g.side32[1], ri.y);
-    F.pi.z = fmaf((float)e[2], g.side32[2], ri.z);
-  } else {
-    F.pi.x = F.valid ? a.pos[F.pidx] : 0.0;
-    F.pi.y = F.valid ? a.pos[a.n + F.pidx] : 0.0;
-    F.pi.z = F.valid ? a.pos[2 * a.n + F.pidx] : 0.0;
-    if (a.n_drift > 0 && F.valid) {  // drifted since the sort: the image nearest its sorted subtile
-      F.pi.x += g.box * rint(((gi[0] + 0.5) * g.side64[0] - F.pi.x) / g.box);
-      F.pi.y += g.box * rint(((gi[1] + 0.5) * g.side64[1] - F.pi.y) / g.box);
-      F.pi.z += g.box * rint(((gi[2] + 0.5) * g.side64[2] - F.pi.z) / g.box);
-    }
-  }
-  const Real big = Real(1e30);
-  F.lo.x = warp_min(F.valid ? F.pi.x : big);
-  F.lo.y = warp_min(F.valid ? F.pi.y : big);
-  F.lo.z = warp_min(F.valid ? F.pi.z : big);
-  F.hi.x = warp_max(F.valid ? F.pi.x : -big);
-  F.hi.y = warp_max(F.valid ? F.pi.y : -big);
-  F.hi.z = warp_max(F.valid ? F.pi.z : -big);
-  if (!F.valid) { F.pi.x = big; F.pi.y = big; F.pi.z = big; }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    F.elo[d] = __reduce_min_sync(full, F.valid ? e[d] : 1 << 20) - rc.R[d];
-    int ehi = __reduce_max_sync(full, F.valid ? e[d] : -(1 << 20)) + rc.R[d];
-    F.ext[d] = ehi - F.elo[d] + 1;
-    if constexpr (sizeof(Real) == 4) F.org[d] = 0.0f;
-    else F.org[d] = (double)F.g0[d] * g.side64[d];
-  }
-  F.inv_ext[0] = 1.0f / (float)F.ext[2];
-  F.inv_ext[1] = 1.0f / (float)F.ext[1];
-}
-
-#ifndef P3M_FAST_DECODE
-#define P3M_FAST_DECODE 1  // candidate decoding and subtile encoding without integer division
-#endif
-
-// Candidate subtile cc (of ncand) of the blocky ball around the chunk's subtile
-// block: whether its box gap to the receivers' bounding box is below the reach
-// and it holds particles at indices >= clip_from; if so their range and the
-// subtile offset.
-template <class Real>
-__device__ __forceinline__ bool candidate_range(const TraversalArgs& a, const Reach& rc, const ChunkFrame<Real>& F,
-                                                int cc, int ncand, int clip_from, int& start, int& cnt,
-                                                unsigned& dpk) {
-  const Geometry& g = a.g;
-  start = 0;
-  cnt = 0;
-  dpk = 0;
-  if (cc >= ncand) return false;
-  int t, dx;
-  if (P3M_FAST_DECODE && ncand < (1 << 22)) {  // always, unless a drift has widened the block enormously
-    t = quot_small(cc, F.ext[2], F.inv_ext[0]);
-    dx = quot_small(t, F.ext[1], F.inv_ext[1]);
-  } else {
-    t = cc / F.ext[2];
-    dx = t / F.ext[1];
-  }
-  int dz = cc - t * F.ext[2];
-  int dy = t - dx * F.ext[1];
-  dx += F.elo[0]; dy += F.elo[1]; dz += F.elo[2];
-  const int dd[3] = {dx, dy, dz};
-  const Real blo[3] = {F.lo.x, F.lo.y, F.lo.z}, bhi[3] = {F.hi.x, F.hi.y, F.hi.z};
-  Real gap2 = Real(0);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Real side;
-    if constexpr (sizeof(Real) == 4) side = g.side32[d]; else side = g.side64[d];
-    Real jlo = F.org[d] + Real(dd[d]) * side;
-    Real jhi = jlo + side;
-    Real gp = fmax(fmax(blo[d] - jhi, jlo - bhi[d]), Real(0));
-    gap2 += gp * gp;
-  }
-  Real sub2;
-  if constexpr (sizeof(Real) == 4) sub2 = rc.sub2; else sub2 = rc.sub2_d;
-  if (!(gap2 < sub2)) return false;
-  int gx = F.g0[0] + dx, gy = F.g0[1] + dy, gz = F.g0[2] + dz;
-  gx += gx < 0 ? g.M[0] : (gx >= g.M[0] ? -g.M[0] : 0);
-  gy += gy < 0 ? g.M[1] : (gy >= g.M[1] ? -g.M[1] : 0);
-  gz += gz < 0 ? g.M[2] : (gz >= g.M[2] ? -g.M[2] : 0);
-  const int sid = P3M_FAST_DECODE ? encode_subtile_fast(g, gx, gy, gz) : encode_subtile(g, gx, gy, gz);
-  start = max(a.offsets[sid], clip_from);
-  cnt = a.offsets[sid + 1] - start;
-  dpk = pack_delta(dx, dy, dz);
-  return cnt > 0;
-}
-
-// Append the taken candidates of one round (ballot tm) to the warp's list.
-__device__ __forceinline__ void append_round(WarpList& L, int lane, bool take, int start, int cnt, unsigned dpk,
-                                             unsigned tm, int& nlist, int& total) {
-  const unsigned full = 0xffffffffu;
-  int v = take ? cnt : 0;  // inclusive scan of the taken counts
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int u = __shfl_up_sync(full, v, o);
-    if (lane >= o) v += u;
-  }
-  const int round_total = __shfl_sync(full, v, 31);
-  if (take) {
-    const int slot = nlist + __popc(tm & ((1u << lane) - 1u));
-    L.start[slot] = start;
-    L.pre[slot] = total + v - cnt;
-    L.delta[slot] = dpk;
-  }
-  nlist += __popc(tm);
-  total += round_total;
-}
-
-// Enumerate the subtiles of the blocky ball around the chunk's subtile block
-// (32 candidates per round, one per lane), keep those whose box gap to the
-// receivers' bounding box is below x_r and that hold particles, and append their
-// particle ranges to the warp's list; `proc(nlist, total)` consumes a full list.
-// With nparts > 1 only every nparts-th candidate subtile, starting at `part`, is
-// enumerated: the parts of a chunk split its suppliers between work items.
-template <class Real, class Proc>
-__device__ __forceinline__ void enumerate_suppliers(const TraversalArgs& a, const Reach& rc, const ChunkFrame<Real>& F,
-                                                    WarpList& L, int lane, int part, int nparts, Proc&& proc) {
-  const unsigned full = 0xffffffffu;
-  const int ncand_all = F.ext[0] * F.ext[1] * F.ext[2];
-  const int ncand = (ncand_all - part + nparts - 1) / nparts;  // candidates of this part
-  int nlist = 0, total = 0;
-  for (int cb = 0; cb < ncand; cb += kWarp) {
-    int start, cnt;
-    unsigned dpk;
-    const bool take = candidate_range<Real>(a, rc, F, (cb + lane) * nparts + part, ncand_all, 0, start, cnt, dpk);
-    const unsigned tm = __ballot_sync(full, take);
-    if (tm == 0) continue;
-    if (nlist + __popc(tm) > kListCap) {
-      __syncwarp();
-      proc(nlist, total);
-      __syncwarp();
-      nlist = 0;
-      total = 0;
-    }
-    append_round(L, lane, take, start, cnt, dpk, tm, nlist, total);
-  }
-  __syncwarp();
-  if (nlist > 0) proc(nlist, total);
-  __syncwarp();
-}
-
-// As enumerate_suppliers, with the ranges cut to indices >= clip_from, and
-// `proc(nlist, total, last)` called from one place: each time the list fills up
-// and once more at the end (last = true, possibly with an empty list), so that
-// a large consumer is inlined once.
-template <class Real, class Proc>
-__device__ __forceinline__ void enumerate_suppliers_once(const TraversalArgs& a, const Reach& rc,
-                                                         const ChunkFrame<Real>& F, WarpList& L, int lane,
-                                                         int clip_from, Proc&& proc) {
-  const unsigned full = 0xffffffffu;
-  const int ncand = F.ext[0] * F.ext[1] * F.ext[2];
-  int nlist = 0, total = 0;
-  int cb = 0;
-  bool take = false;
-  int start = 0, cnt = 0;
-  unsigned dpk = 0, tm = 0;
-  for (;;) {
-    bool overflow = false;
-    for (; cb < ncand; cb += kWarp) {
-      take = candidate_range<Real>(a, rc, F, cb + lane, ncand, clip_from, start, cnt, dpk);
-      tm = __ballot_sync(full, take);
-      if (tm == 0) continue;
-      if (nlist + __popc(tm) > kListCap) {  // flush first; this batch of candidates is appended after
-        overflow = true;
-        break;
-      }
-      append_round(L, lane, take, start, cnt, dpk, tm, nlist, total);
-    }
-    __syncwarp();
-    proc(nlist, total, !overflow);
-    __syncwarp();
-    if (!overflow) break;
-    nlist = 0;
-    total = 0;
-    append_round(L, lane, take, start, cnt, dpk, tm, nlist, total);
-    cb += kWarp;
-  }
-}
-
-// Load supplier number f of the list (lane-parallel): its position in the
-// chunk frame (FP32) or its nearest image in absolute coordinates (FP64),
-// and for the VJP its masked abar.  Returns whether it can reach the receivers'
-// bounding box.
-template <class Real, bool VJP>
+// Supplier number f of the list (lane-parallel): its position in the chunk frame and
+// its masked abar.  Returns whether it can reach the receivers' bounding box.
 __device__ __forceinline__ bool load_supplier(const TraversalArgs& a, const WarpList& L, int nlist, int f,
-                                              const ChunkFrame<Real>& F, Vec3<Real>& pj, Vec3<Real>& aj,
-                                              Real* gap2_out = nullptr) {
+                                              const ChunkFrame& F, Vec3<float>& pj, Vec3<float>& aj, float* gap2_out) {
   int lo_e = 0, hi_e = nlist - 1;  // last entry with pre <= f
   while (lo_e < hi_e) {
     int mid = (lo_e + hi_e + 1) >> 1;
@@ -612,168 +281,24 @@ __device__ __forceinline__ bool load_supplier(const TraversalArgs& a, const Warp
   int j = L.start[lo_e] + (f - L.pre[lo_e]);
   int dx, dy, dz;
   unpack_delta(L.delta[lo_e], dx, dy, dz);
-  if constexpr (sizeof(Real) == 4) {
-    float4 r = a.rel4[j];
-    pj.x = fmaf((float)dx, a.g.side32[0], r.x);
-    pj.y = fmaf((float)dy, a.g.side32[1], r.y);
-    pj.z = fmaf((float)dz, a.g.side32[2], r.z);
-    if (VJP) {
-      float4 q = a.abar4[j];
-      aj.x = q.x; aj.y = q.y; aj.z = q.z;
-    }
-  } else {
-    int gx = F.g0[0] + dx, gy = F.g0[1] + dy, gz = F.g0[2] + dz;
-    double sx = gx < 0 ? -a.g.box : (gx >= a.g.M[0] ? a.g.box : 0.0);
-    double sy = gy < 0 ? -a.g.box : (gy >= a.g.M[1] ? a.g.box : 0.0);
-    double sz = gz < 0 ? -a.g.box : (gz >= a.g.M[2] ? a.g.box : 0.0);
-    pj.x = a.pos[j] + sx;
-    pj.y = a.pos[a.n + j] + sy;
-    pj.z = a.pos[2 * a.n + j] + sz;
-    if (a.n_drift > 0) {  // drifted since the sort: the image nearest the candidate subtile
-      pj.x += a.g.box * rint(((gx + 0.5) * a.g.side64[0] - pj.x) / a.g.box);
-      pj.y += a.g.box * rint(((gy + 0.5) * a.g.side64[1] - pj.y) / a.g.box);
-      pj.z += a.g.box * rint(((gz + 0.5) * a.g.side64[2] - pj.z) / a.g.box);
-    }
-    if (VJP) {
-      aj.x = a.abar_d[j]; aj.y = a.abar_d[a.n + j]; aj.z = a.abar_d[2 * a.n + j];
-    }
-  }
-  Real tx = fmax(fmax(F.lo.x - pj.x, pj.x - F.hi.x), Real(0));
-  Real ty = fmax(fmax(F.lo.y - pj.y, pj.y - F.hi.y), Real(0));
-  Real tz = fmax(fmax(F.lo.z - pj.z, pj.z - F.hi.z), Real(0));
-  const Real gap2 = tx * tx + ty * ty + tz * tz;
-  if (gap2_out) *gap2_out = gap2;
-  return gap2 < Real(a.f.margin2_f);
+  float4 r = a.rel4[j];
+  pj.x = fmaf((float)dx, a.g.side32[0], r.x);
+  pj.y = fmaf((float)dy, a.g.side32[1], r.y);
+  pj.z = fmaf((float)dz, a.g.side32[2], r.z);
+  float4 q = a.abar4[j];
+  aj.x = q.x; aj.y = q.y; aj.z = q.z;
+  const float gap2 = box_gap2(F, pj);
+  *gap2_out = gap2;
+  return gap2 < a.f.margin2_f;
 }
 
-// Generic path (FP64 forward, and the adjoint in both precisions): every
-// surviving supplier is broadcast with shuffles and evaluated by all lanes.
-template <class Real, bool VJP, int SOFT>
-__device__ __forceinline__ void process_list(const TraversalArgs& a, const WarpList& L, int nlist, int total, int lane,
-                                             const ChunkFrame<Real>& F, const Vec3<Real>& abar_i, Vec3<Real>& acc,
-                                             int& hits) {
-  const unsigned full = 0xffffffffu;
-  for (int b = 0; b < total; b += kWarp) {
-    int f = b + lane;
-    Vec3<Real> pj = {Real(0), Real(0), Real(0)};
-    Vec3<Real> aj = {Real(0), Real(0), Real(0)};
-    bool keep = false;
-    if (f < total) keep = load_supplier<Real, VJP>(a, L, nlist, f, F, pj, aj);
-    unsigned m = __ballot_sync(full, keep);
-    while (m) {
-      int src = __ffs(m) - 1;
-      m &= m - 1;
-      Real xj = __shfl_sync(full, pj.x, src);
-      Real yj = __shfl_sync(full, pj.y, src);
-      Real zj = __shfl_sync(full, pj.z, src);
-      Real dx = F.pi.x - xj, dy = F.pi.y - yj, dz = F.pi.z - zj;
-      Real r2 = dx * dx + dy * dy + dz * dz;
-      bool hit;
-      if constexpr (sizeof(Real) == 4) hit = r2 < a.f.xr2_f; else hit = r2 < a.f.xr2_d;
-      Vec3<Real> vj;
-      if (VJP) {
-        vj.x = __shfl_sync(full, aj.x, src);
-        vj.y = __shfl_sync(full, aj.y, src);
-        vj.z = __shfl_sync(full, aj.z, src);
-      }
-      if (__any_sync(full, hit)) {
-        Real B, D = Real(0);
-        if constexpr (sizeof(Real) == 4) {
-          float Dm = 0.f;
-          B = bracket_main_f32<SOFT, VJP>(r2, a.f, Dm);
-          D = Dm;
-          // forward: a zero displacement contributes nothing, so r = 0 skips the
-          // softened branch; the VJP needs B(0) for coincident distinct particles
-          bool rare = hit && (r2 < a.f.rsw2_f) && (VJP || r2 > 0.0f);
-          if (__any_sync(full, rare)) {
-            float Ds = 0.f;
-            float Bs = bracket_soft_f32<SOFT, VJP>(r2, a.f, a.sc, Ds);
-            if (rare) { B = Bs; D = Ds; }
-          }
-        } else {
-          B = (hit && (VJP || r2 > 0.0)) ? bracket_f64<SOFT, VJP>(r2, a.f, a.sc, D) : 0.0;
-        }
-        if (!hit || (!VJP && r2 == Real(0))) { B = Real(0); D = Real(0); }
-        if (VJP) {
-          Real vx = abar_i.x - vj.x, vy = abar_i.y - vj.y, vz = abar_i.z - vj.z;
-          Real c = D * (dx * vx + dy * vy + dz * vz);
-          acc.x += B * vx + c * dx;
-          acc.y += B * vy + c * dy;
-          acc.z += B * vz + c * dz;
-        } else {
-          acc.x += B * dx;
-          acc.y += B * dy;
-          acc.z += B * dz;
-        }
-        hits += hit ? 1 : 0;
-      }
-    }
-  }
-}
-
-template <class Real>
-__device__ __forceinline__ void store_result(const TraversalArgs& a, const ChunkFrame<Real>& F, const Vec3<Real>& acc) {
+__device__ __forceinline__ void store_result(const TraversalArgs& a, const ChunkFrame& F, const Vec3<float>& acc) {
   if (!F.valid) return;
-  const Real s = -Real(a.f.G_m);
-  Real* o = (Real*)a.out;
+  const float s = -(float)a.f.G_m;
+  float* o = (float*)a.out;
   o[F.pidx] = s * acc.x;
   o[a.n + F.pidx] = s * acc.y;
   o[2 * a.n + F.pidx] = s * acc.z;
-}
-
-__device__ __forceinline__ int next_chunk(const TraversalArgs& a, int lane) {
-  int c = 0;
-  if (lane == 0) c = atomicAdd(a.counter, 1);
-  return __shfl_sync(0xffffffffu, c, 0);
-}
-
-// The c-th chunk to process (c < n_chunks): the chunk list is in the sorted, spatial
-// order, which keeps neighbouring chunks, and the suppliers they share, together in L2.
-__device__ __forceinline__ Chunk chunk_at(const TraversalArgs& a, int c) { return a.chunks[c]; }
-
-// Work items per chunk of the one-sided kernel: with few chunks (sparse receivers,
-// the deepest rungs) each chunk's candidate subtiles are split between up to
-// kMaxParts work items so that every resident warp has work; their partial sums
-// are added in a fixed order by k_parts_finish.
-__host__ __device__ __forceinline__ int parts_for(int n_chunks) {
-  if (n_chunks <= 0) return 1;
-  const int k = kPartItems / n_chunks;
-  return k < 1 ? 1 : (k > kMaxParts ? kMaxParts : k);
-}
-
-template <class Real, bool VJP, int SOFT>
-__global__ void __launch_bounds__(kForceThreads) k_traverse(TraversalArgs a) {
-  __shared__ WarpList lists[kForceWarps];
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  WarpList& L = lists[threadIdx.x >> 5];
-  const int n_chunks = *a.n_chunks;
-  const Reach rc = make_reach(a);
-  unsigned long long pair_total = 0;
-  for (;;) {
-    const int c = next_chunk(a, lane);
-    if (c >= n_chunks) break;
-    ChunkFrame<Real> F;
-    load_chunk<Real>(a, rc, chunk_at(a, c), lane, F);
-    Vec3<Real> abar_i = {Real(0), Real(0), Real(0)};
-    if (VJP && F.valid) {
-      if constexpr (sizeof(Real) == 4) {
-        float4 q = a.abar4[F.pidx];
-        abar_i.x = q.x; abar_i.y = q.y; abar_i.z = q.z;
-      } else {
-        abar_i.x = a.abar_d[F.pidx]; abar_i.y = a.abar_d[a.n + F.pidx]; abar_i.z = a.abar_d[2 * a.n + F.pidx];
-      }
-    }
-    Vec3<Real> acc = {Real(0), Real(0), Real(0)};
-    int hits = 0;
-    enumerate_suppliers<Real>(a, rc, F, L, lane, 0, 1, [&](int nlist, int total) {
-      process_list<Real, VJP, SOFT>(a, L, nlist, total, lane, F, abar_i, acc, hits);
-    });
-    store_result<Real>(a, F, acc);
-    if (F.valid) hits -= 1;  // the receiver met itself once (r = 0)
-    pair_total += (unsigned long long)__reduce_add_sync(full, (unsigned)hits);
-  }
-  if (lane == 0 && pair_total) atomicAdd(a.pairs, pair_total);
 }
 
 // ---------------------------------------------------------------------------
@@ -796,14 +321,6 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-
-// cp.async of 16 bytes into shared memory (completion per thread, by commit groups)
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 // As P3M_SYM_CPASYNC for the one-sided kernel (2.087 -> 2.052 ms all active on the
 // 128^3 set).
@@ -847,7 +364,7 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
   const int lane = threadIdx.x & 31;
   PackedSmem& S = smem[threadIdx.x >> 5];
   const int n_chunks = *a.n_chunks;
-  const int nparts = a.part_acc ? parts_for(n_chunks) : 1;
+  const int nparts = a.part_acc ? parts_for(n_chunks, a.part_items, kMaxParts) : 1;
   const int n_items = n_chunks * nparts;
   const Reach rc = make_reach(a);
   const float xr2 = a.f.xr2_f;
@@ -857,33 +374,17 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
     const int w = next_chunk(a, lane);
     if (w >= n_items) break;
     const int c = w / nparts, part = w - c * nparts;
-    ChunkFrame<float> F;
-    load_chunk<float>(a, rc, chunk_at(a, c), lane, F);
+    ChunkFrame F;
+    load_chunk(a, rc, chunk_at(a, c), lane, F);
     const f2 px = pk(F.pi.x, F.pi.x), py = pk(F.pi.y, F.pi.y), pz = pk(F.pi.z, F.pi.z);
     f2 ax = pk(0.f, 0.f), ay = pk(0.f, 0.f), az = pk(0.f, 0.f);
     f2 hitsf = pk(0.f, 0.f);  // interacting pairs of this lane (exact integers in FP32)
-    enumerate_suppliers<float>(a, rc, F, S.L, lane, part, nparts, [&](int nlist, int total) {
+    enumerate_strided(a, rc, F, S.L, lane, part, nparts, [&](int nlist, int total) {
       float* sxy = (float*)S.sxy;
       float* sz = (float*)S.sz;
       const WarpList& L = S.L;
-      // Supplier f = b + lane of batch b lies in list entry e_cur + (number of
-      // entries starting in (b, b + lane]); the start positions of the next 32
-      // entries are gathered into one bit mask with a warp OR-reduction.
-      int e_cur = 0;  // entry holding position b
-      auto locate = [&](int b, int& j, unsigned& dpk) -> bool {
-        const int ek = e_cur + 1 + lane;
-        const int pos = (ek < nlist) ? L.pre[ek] - b : 64;
-        const unsigned bit = (pos > 0 && pos < kWarp) ? (1u << pos) : 0u;
-        const unsigned starts = __reduce_or_sync(full, bit);
-        const bool at_end = __any_sync(full, pos == kWarp);
-        const unsigned upto = (lane == kWarp - 1) ? 0xffffffffu : ((2u << lane) - 1u);
-        const int e = e_cur + __popc(starts & upto);
-        e_cur += __popc(starts) + (at_end ? 1 : 0);
-        const bool have = b + lane < total;
-        j = have ? L.start[e] + (b + lane - L.pre[e]) : 0;
-        dpk = have ? L.delta[e] : 0u;
-        return have;
-      };
+      ListCursor<WarpList> cur;
+      auto locate = [&](int b, int& j, unsigned& dpk) { return cur.locate(L, nlist, total, lane, b, j, dpk); };
       // software pipeline: the record of batch b + 32 is loaded while batch b is evaluated
       int jn;
       unsigned dn;
@@ -1014,7 +515,7 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
     acc.y = l + h;
     upk(az, l, h);
     acc.z = l + h;
-    if (nparts == 1) store_result<float>(a, F, acc);
+    if (nparts == 1) store_result(a, F, acc);
     else a.part_acc[(int64_t)w * kWarp + lane] = make_float4(acc.x, acc.y, acc.z, 0.f);
     upk(hitsf, l, h);
     // the receiver met itself once (r = 0), in the part that holds its own subtile; every
@@ -1031,7 +532,7 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
 // split its chunks (nothing to do otherwise).  One warp per chunk position.
 __global__ void k_parts_finish(TraversalArgs a) {
   const int n_chunks = *a.n_chunks;
-  const int nparts = parts_for(n_chunks);
+  const int nparts = parts_for(n_chunks, a.part_items, kMaxParts);
   if (nparts == 1) return;
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1125,6 +626,15 @@ constexpr int kSymUnroll = P3M_SYM_UNROLL;
 #define P3M_SYMV_MINBLOCKS 6  // the adjoint instance
 #endif
 
+#ifndef P3M_SYM_ITEMS
+#define P3M_SYM_ITEMS 0
+#endif
+#ifndef P3M_SYM_PARTS
+#define P3M_SYM_PARTS 8
+#endif
+constexpr int kSymItems = P3M_SYM_ITEMS;
+constexpr int kSymMaxParts = P3M_SYM_PARTS;
+
 __device__ __forceinline__ f2 shfl2(f2 v, int src) {
   f2 r;
   r.v = __shfl_sync(0xffffffffu, v.v, src);
@@ -1157,16 +667,19 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
     vzf = (float*)S.vz;
   }
   const int n_chunks = *a.n_chunks;
+  const int nparts = parts_for(n_chunks, kSymItems, kSymMaxParts);
+  const int n_items = n_chunks * nparts;
   const Reach rc = make_reach(a);
   const float xr2 = a.f.xr2_f;
   const float xr2s = xr2 * kCutScale;
   unsigned long long pair_total = 0;
   for (;;) {
-    const int c = next_chunk(a, lane);
-    if (c >= n_chunks) break;
+    const int w = next_chunk(a, lane);
+    if (w >= n_items) break;
+    const int c = w / nparts, part = w - c * nparts;
     const Chunk ch = chunk_at(a, c);
-    ChunkFrame<float> F;
-    load_chunk<float>(a, rc, ch, lane, F);
+    ChunkFrame F;
+    load_chunk(a, rc, ch, lane, F);
     const int i_self = F.valid ? F.pidx : 0x7fffffff;  // the mask j > i is false on empty lanes
     const int c_end = ch.start + ch.count;
     const float rx = F.valid ? F.pi.x : kSymPad, ry = F.valid ? F.pi.y : kSymPad, rz = F.valid ? F.pi.z : kSymPad;
@@ -1458,7 +971,7 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
     // comes back by a shuffle from lane l - k.  The staged suppliers then start after
     // the chunk, so no block needs the j > i mask.
     constexpr bool kOwnTri = !VJP && P3M_SYM_OWN_TRIANGLE;
-    if constexpr (kOwnTri) {
+    if (kOwnTri && part == 0) {
       float ox = 0.f, oy = 0.f, oz = 0.f, oh = 0.f;
 #pragma unroll 1
       for (int k = 1; k <= kWarp / 2; ++k) {
@@ -1494,28 +1007,16 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
     // Stage the survivors of each batch of 32 list positions; evaluate a block
     // whenever 64 are staged, and the rest once the enumeration is done (one
     // call site of eval_block, so its loops are inlined once).
-    enumerate_suppliers_once<float>(
-        a, rc, F, S.L, lane, kOwnTri ? c_end : ch.start,
-        [&](int nlist, int total, bool last) {
+    enumerate_suppliers(
+        a, rc, F, S.L, lane, part, nparts, kOwnTri ? c_end : ch.start,
+        [&](int nlist, int lo, int hi, bool last) {
           const WarpList& L = S.L;
-          int e_cur = 0;  // list entry holding position b (as in k_force_packed)
-          auto locate = [&](int b, int& j, unsigned& dpk) -> bool {
-            const int ek = e_cur + 1 + lane;
-            const int pos = (ek < nlist) ? L.pre[ek] - b : 64;
-            const unsigned bit = (pos > 0 && pos < kWarp) ? (1u << pos) : 0u;
-            const unsigned starts = __reduce_or_sync(full, bit);
-            const bool at_end = __any_sync(full, pos == kWarp);
-            const unsigned upto = (lane == kWarp - 1) ? 0xffffffffu : ((2u << lane) - 1u);
-            const int e = e_cur + __popc(starts & upto);
-            e_cur += __popc(starts) + (at_end ? 1 : 0);
-            const bool have = b + lane < total;
-            j = have ? L.start[e] + (b + lane - L.pre[e]) : 0;
-            dpk = have ? L.delta[e] : 0u;
-            return have;
-          };
+          ListCursor<WarpList> cur;
+          cur.seek(L, nlist, lane, lo);
+          auto locate = [&](int b, int& j, unsigned& dpk) { return cur.locate(L, nlist, hi, lane, b, j, dpk); };
           int jn;
           unsigned dn;
-          bool vn = locate(0, jn, dn);
+          bool vn = locate(lo, jn, dn);
 #if P3M_SYM_CPASYNC
           int buf = 0;
           if (vn) cp_async16(&S.rec[0][lane], a.rel4 + jn);
@@ -1526,8 +1027,8 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
 #endif
           float4 an = make_float4(0.f, 0.f, 0.f, 0.f);
           if (VJP && vn) an = a.abar4[jn];
-          for (int b = 0;; b += kWarp) {
-            const bool more = b < total;  // warp-uniform
+          for (int b = lo;; b += kWarp) {
+            const bool more = b < hi;  // warp-uniform
             bool keep = false, near = false, own = false;
             Vec3<float> pj = {0.f, 0.f, 0.f};
             int j = 0, rank = 0, ns = 0;
@@ -1537,7 +1038,7 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
               const unsigned dpk = dn;
               j = jn;
               if (VJP) aj = an;
-              vn = (b + kWarp < total) ? locate(b + kWarp, jn, dn) : false;
+              vn = (b + kWarp < hi) ? locate(b + kWarp, jn, dn) : false;
 #if P3M_SYM_CPASYNC
               if (vn) cp_async16(&S.rec[buf ^ 1][lane], a.rel4 + jn);
               cp_async_commit();
@@ -1643,15 +1144,15 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_vjp_packed(Trav
   for (;;) {
     const int c = next_chunk(a, lane);
     if (c >= n_chunks) break;
-    ChunkFrame<float> F;
-    load_chunk<float>(a, rc, chunk_at(a, c), lane, F);
+    ChunkFrame F;
+    load_chunk(a, rc, chunk_at(a, c), lane, F);
     const f2 px = pk(F.pi.x, F.pi.x), py = pk(F.pi.y, F.pi.y), pz = pk(F.pi.z, F.pi.z);
     float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
     if (F.valid) ab = a.abar4[F.pidx];
     const f2 vix = pk(ab.x, ab.x), viy = pk(ab.y, ab.y), viz = pk(ab.z, ab.z);
     f2 gx = pk(0.f, 0.f), gy = pk(0.f, 0.f), gz = pk(0.f, 0.f);
     int hits = 0;
-    enumerate_suppliers<float>(a, rc, F, S.L, lane, 0, 1, [&](int nlist, int total) {
+    enumerate_strided(a, rc, F, S.L, lane, 0, 1, [&](int nlist, int total) {
       float* sxy = (float*)S.sxy;
       float* sz = (float*)S.sz;
       float* vxy = (float*)S.vxy;
@@ -1662,7 +1163,7 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_vjp_packed(Trav
         bool keep = false, near = false;
         if (f < total) {
           float gap2;
-          keep = load_supplier<float, true>(a, S.L, nlist, f, F, pj, aj, &gap2);
+          keep = load_supplier(a, S.L, nlist, f, F, pj, aj, &gap2);
           near = keep && gap2 < a.f.rsw2_f;  // may come within r_sw of a receiver (or coincide)
         }
         const unsigned m = __ballot_sync(full, keep);
@@ -1757,7 +1258,7 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_vjp_packed(Trav
     acc.y = l + h;
     upk(gz, l, h);
     acc.z = l + h;
-    store_result<float>(a, F, acc);
+    store_result(a, F, acc);
     hits = F.valid ? hits - 1 : 0;  // the receiver met itself once (r = 0)
     pair_total += (unsigned long long)__reduce_add_sync(full, (unsigned)hits);
   }
@@ -1789,34 +1290,29 @@ static SeriesConsts make_series() {
   return s;
 }
 
-template <class Real, bool VJP, int SOFT>
-static cudaError_t launch_traverse(p3m_sr_ctx* ctx, const TraversalArgs& a) {
-  constexpr bool packed = (sizeof(Real) == 4);  // FP32: packed broadcast kernels
+// One-sided FP32 kernels.
+template <bool VJP, int SOFT>
+static cudaError_t launch_packed(p3m_sr_ctx* ctx, const TraversalArgs& a) {
   static int blocks_per_sm = 0;
   if (blocks_per_sm == 0) {
-    if (packed && !VJP)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_force_packed<SOFT>, kPThreads, 0);
-    else if (packed)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_vjp_packed<SOFT>, kPThreads, 0);
-    else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_traverse<Real, VJP, SOFT>, kForceThreads, 0);
+    if (VJP) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_vjp_packed<SOFT>, kPThreads, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_force_packed<SOFT>, kPThreads, 0);
     if (blocks_per_sm < 1) blocks_per_sm = 1;
   }
   unsigned grid = (unsigned)(ctx->num_sms * blocks_per_sm);
   const int slot = VJP ? 1 : 0;
   TraversalArgs ap = a;
-  if (packed && !VJP) ap.part_acc = ctx->part_acc;  // sparse receivers: chunks split into parts
+  if (!VJP) {  // sparse receivers: chunks split into parts
+    ap.part_acc = ctx->part_acc;
+    ap.part_items = ctx->part_items;
+  }
   cudaEventRecord(ctx->kt_ev[2 * slot], ctx->stream);
-  if (packed && !VJP)
-    k_force_packed<SOFT><<<grid, kPThreads, 0, ctx->stream>>>(ap);
-  else if (packed)
-    k_vjp_packed<SOFT><<<grid, kPThreads, 0, ctx->stream>>>(ap);
-  else
-    k_traverse<Real, VJP, SOFT><<<grid, kForceThreads, 0, ctx->stream>>>(ap);
+  if (VJP) k_vjp_packed<SOFT><<<grid, kPThreads, 0, ctx->stream>>>(ap);
+  else k_force_packed<SOFT><<<grid, kPThreads, 0, ctx->stream>>>(ap);
   ++ctx->launches;
   cudaEventRecord(ctx->kt_ev[2 * slot + 1], ctx->stream);
   ctx->kt_pending[slot] = true;
-  if (packed && !VJP) {
+  if (!VJP) {
     k_parts_finish<<<(unsigned)(ctx->num_sms * 4), 256, 0, ctx->stream>>>(ap);
     ++ctx->launches;
   }
@@ -1857,12 +1353,12 @@ static cudaError_t launch_sym(p3m_sr_ctx* ctx, const TraversalArgs& a) {
   }
 }
 
-template <class Real, bool VJP>
-static cudaError_t dispatch_traverse(p3m_sr_ctx* ctx, const TraversalArgs& a) {
+template <bool VJP>
+static cudaError_t dispatch_packed(p3m_sr_ctx* ctx, const TraversalArgs& a) {
   switch (ctx->prm.softening) {
-    case P3M_SOFT_NONE: return launch_traverse<Real, VJP, P3M_SOFT_NONE>(ctx, a);
-    case P3M_SOFT_PLUMMER: return launch_traverse<Real, VJP, P3M_SOFT_PLUMMER>(ctx, a);
-    default: return launch_traverse<Real, VJP, P3M_SOFT_BSPLINE>(ctx, a);
+    case P3M_SOFT_NONE: return launch_packed<VJP, P3M_SOFT_NONE>(ctx, a);
+    case P3M_SOFT_PLUMMER: return launch_packed<VJP, P3M_SOFT_PLUMMER>(ctx, a);
+    default: return launch_packed<VJP, P3M_SOFT_BSPLINE>(ctx, a);
   }
 }
 
@@ -1901,9 +1397,9 @@ static TraversalArgs base_args(p3m_sr_ctx* ctx) {
   a.f = ctx->fc;
   a.sc = series;
   a.offsets = ctx->offsets;
-  a.cell = ctx->cell;
   a.n = ctx->n;
   a.rel4 = ctx->rel4;
+  a.rel_scale = 1.0f;
   a.pairs = ctx->pair_count;
   a.drift_slots = ctx->drift_slots;
   a.n_drift = ctx->n_drift;
@@ -1969,7 +1465,7 @@ extern "C" p3m_status p3m_sr_forces(p3m_sr_ctx* ctx, const double* pos, int prec
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->pair_count, 0, sizeof(unsigned long long), s), "memset")) != P3M_OK)
     return st;
   if (ctx->n == 0) return P3M_OK;
-  if (precision == 32 && (st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
+  if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 3, 0, sizeof(int), s), "memset")) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
@@ -1979,8 +1475,8 @@ extern "C" p3m_status p3m_sr_forces(p3m_sr_ctx* ctx, const double* pos, int prec
   a.active_idx = ctx->all_active ? nullptr : ctx->active_idx;
   a.out = acc_out;
   cudaError_t e;
-  if (precision == 32 && ctx->all_active && ctx->symmetric) e = launch_sym<false>(ctx, a);
-  else e = (precision == 32) ? dispatch_traverse<float, false>(ctx, a) : dispatch_traverse<double, false>(ctx, a);
+  if (precision == 64) e = launch_pair64(ctx, a, false);
+  else e = ctx->all_active && ctx->symmetric ? launch_sym<false>(ctx, a) : dispatch_packed<false>(ctx, a);
   if ((st = cuda_check(ctx, e, "force kernel")) != P3M_OK) return st;
   report_latched(ctx);
   return P3M_OK;
@@ -2058,6 +1554,7 @@ extern "C" p3m_status p3m_sr_forces_tabulated(p3m_sr_ctx* ctx, const double* pos
   a.out = acc_out;
   a.table = ctx->table;
   a.part_acc = ctx->part_acc;
+  a.part_items = ctx->part_items;
   a.n_table = nt;
   a.table_scale = (float)(nt / (ctx->prm.x_r * ctx->prm.x_r));
   const size_t shm = sizeof(float) * nt;
@@ -2109,7 +1606,7 @@ extern "C" p3m_status p3m_sr_vjp(p3m_sr_ctx* ctx, const double* pos, int precisi
       return st;
   }
   if ((st = ensure_all_chunks(ctx)) != P3M_OK) return st;
-  if (precision == 32 && (st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
+  if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
   if (precision == 32)
     k_abar_f32<<<blocks_for(n, 256), 256, 0, s>>>((const float*)acc_bar, ctx->active_flag, ctx->all_active, n,
                                                    ctx->abar4);
@@ -2129,8 +1626,8 @@ extern "C" p3m_status p3m_sr_vjp(p3m_sr_ctx* ctx, const double* pos, int precisi
   a.abar4 = ctx->abar4;
   a.abar_d = ctx->abar_d;
   cudaError_t e;
-  if (precision == 32 && ctx->symmetric) e = launch_sym<true>(ctx, a);  // each pair once (any active set)
-  else e = (precision == 32) ? dispatch_traverse<float, true>(ctx, a) : dispatch_traverse<double, true>(ctx, a);
+  if (precision == 64) e = launch_pair64(ctx, a, true);
+  else e = ctx->symmetric ? launch_sym<true>(ctx, a) : dispatch_packed<true>(ctx, a);  // each pair once (any active set)
   if ((st = cuda_check(ctx, e, "vjp kernel")) != P3M_OK) return st;
   report_latched(ctx);
   return P3M_OK;
@@ -2352,8 +1849,8 @@ extern "C" p3m_status p3m_sr_forces_noalloc(const p3m_sr_params* params, void* c
   a.sc = series;
   a.pos = spos;
   a.rel4 = rel4;
+  a.rel_scale = 1.0f;
   a.offsets = offsets;
-  a.cell = cell;
   a.chunks = chunks;
   a.n_chunks = small + 0;
   a.counter = small + 1;

@@ -402,7 +402,8 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->act_scan, n + 1);
   P3M_ALLOC(ctx->active_idx, n);
   P3M_ALLOC(ctx->tile_chunks, ctx->n_tiles + 1);
-  P3M_ALLOC(ctx->part_acc, std::min<int64_t>(kPartItems, ctx->max_chunks * kMaxParts) * kChunk);
+  ctx->part_items = (int)std::min<int64_t>(kPartItems, ctx->max_chunks * kPartItemsPerChunk);
+  P3M_ALLOC(ctx->part_acc, (int64_t)ctx->part_items * kChunk);
   P3M_ALLOC(ctx->chunks, ctx->max_chunks);
   P3M_ALLOC(ctx->chunks_all, ctx->max_chunks);
   P3M_ALLOC(ctx->dev_small, 16);
@@ -410,6 +411,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->rel4, n);
   P3M_ALLOC(ctx->org, origin_count(ctx->geo));
   ctx->org_cap = origin_count(ctx->geo);
+  P3M_ALLOC(ctx->tab64, pair_table_doubles());
   P3M_ALLOC(ctx->err_dev, 1);
   P3M_ALLOC(ctx->drift_slots, kMaxDrifts);
 #undef P3M_ALLOC
@@ -441,6 +443,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
                        "memset")) != P3M_OK)
     goto fail_alloc;
   if ((st = fill_origins(ctx)) != P3M_OK) goto fail_alloc;
+  if ((st = fill_pair_tables(ctx)) != P3M_OK) goto fail_alloc;
   *out = ctx;
   return P3M_OK;
 fail_alloc:
@@ -536,7 +539,7 @@ extern "C" void p3m_sr_destroy(p3m_sr_ctx* ctx) {
                   ctx->scan_scratch, ctx->gather_tmp, ctx->active_flag, ctx->act_scan, ctx->active_idx,
                   ctx->tile_chunks, ctx->part_acc,
                   ctx->chunks, ctx->chunks_all, ctx->dev_small, ctx->pair_count,
-                  ctx->rel4, ctx->org, ctx->abar4, ctx->abar_d, ctx->table, ctx->err_dev, ctx->drift_slots};
+                  ctx->rel4, ctx->org, ctx->abar4, ctx->abar_d, ctx->table, ctx->tab64, ctx->err_dev, ctx->drift_slots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (ctx->err_host) cudaFreeHost(ctx->err_host);
