@@ -322,7 +322,7 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   return d;
 }
 
-// As P3M_SYM_CPASYNC for the one-sided kernel (2.087 -> 2.052 ms all active on the
+// cp.async record copies as in k_force_sym (2.087 -> 2.052 ms all active on the
 // 128^3 set).
 #ifndef P3M_GP_CPASYNC
 #define P3M_GP_CPASYNC 1
@@ -556,84 +556,61 @@ __global__ void k_parts_finish(TraversalArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// FP32 forward with Newton's third law, for calls in which every particle is a
-// receiver.  The paper pairs two neighbouring tiles only once and updates the
-// particles of both (Section 2.1.3); here each unordered pair {i, j} of sorted
-// indices i < j is evaluated once, by the chunk that holds i, and both
-// particles receive their share.  The chunk's supplier ranges are cut to
-// indices >= its first receiver, and suppliers of the chunk itself are masked
-// to j > i.
+// FP32 kernel with Newton's third law: the forward of calls in which every particle
+// is a receiver, and the adjoint (VJP).  The paper pairs two neighbouring tiles only
+// once and updates the particles of both (Section 2.1.3); here each unordered pair
+// {i, j} of sorted indices i < j is evaluated once, by the chunk that holds i, and
+// both particles receive their share.  The chunk's own pairs come first, in a
+// triangular pass (lane l with lanes l + k and l + k + 8); its supplier ranges are
+// then cut to the indices past its last receiver.
 //
-// The survivors of the box test are staged 64 at a time as 32 packed pairs.  A
-// block of P pairs (P a power of two <= 32) takes P steps: at step k, lane l
-// evaluates its receiver against pair (l + k) mod P of its group of P lanes, so
-// that every receiver meets every pair once and no two lanes of a group touch
-// one supplier at the same time.  Each pair's accumulator travels with it from
-// lane to lane by warp shuffles; at the end of the block the groups' partial
-// sums are reduced and added, like the receivers' own sums at the end of the
-// chunk, into an FP32 float4 array with vector atomics.  k_sym_finish scales
-// that array into the caller's 3 x n output.  Pairs closer than r_sw (the
-// softened form) are evaluated in the step: when some lane holds one, one packed
-// softened evaluation serves both halves and each half selects its form
-// (P3M_SYM_SOFT_INLINE; 0 builds the earlier variant, which queues them per warp
-// and evaluates them 32 at a time, one per lane, with atomics to both particles).
+// The survivors of the box test are staged 64 at a time as 32 packed pairs.  Each half
+// of the warp holds all 32 receivers, two per lane (l and l + 16), and takes half of
+// the pairs: P of them (a power of two <= 16) in P steps.  At step k lane l of a group
+// of P lanes evaluates its two receivers against pair (l + k) mod P, so that every
+// receiver meets every pair once and no two lanes of a group touch one supplier at the
+// same time; each pair's accumulator travels with it from lane to lane by warp
+// shuffles.  At the end of the block the groups' partial sums are reduced and added,
+// like the receivers' own sums at the end of the chunk, into an FP32 float4 array with
+// vector atomics.  k_sym_finish scales that array into the caller's 3 x n output.
+// Pairs closer than r_sw (the softened form) are evaluated in the step: when some lane
+// holds one, one packed softened evaluation serves both halves of a pair and each half
+// selects its form.
+//
+// Bound: issue slots and the FP32 pipe (0.385 of the evaluated slots interact).  The
+// rotation's fixed cost, 6 shuffles, 2 shared loads and the loop, is paid per step, so a
+// step carries four (receiver, supplier) slots per lane instead of two: at 128^3 (654 M
+// ordered pairs) the forward takes 1.28 instead of 1.36 ms (1.07 instead of 1.22 G warp
+// instructions, the FP32 pipe 60% busy), the adjoint 1.82 instead of 1.96 ms.
 // ---------------------------------------------------------------------------
 
 constexpr float kSymPad = 1e10f;  // padding supplier at -1e10, invalid receiver at +1e10: finite B, no hit
 
-// Supplier records of the next batch: copied into a per-warp shared-memory double
-// buffer with cp.async while the current batch is staged (1), or prefetched into
-// registers (0).  Measured on the 128^3 set: 1.551 -> 1.518 ms.
-#ifndef P3M_SYM_CPASYNC
-#define P3M_SYM_CPASYNC 1
-#endif
-
 struct SymSmem {
   WarpList L;
-  float4 sxy[kWarp];  // pair q: (-x_a, -x_b, -y_a, -y_b) of suppliers a = q and b = q + P
+  float4 sxy[kWarp];  // pair q: (-x_a, -x_b, -y_a, -y_b) of suppliers a and b
   float2 sz[kWarp];   // (-z_a, -z_b)
   int2 sj[kWarp];     // (j_a, j_b): sorted indices, -1 for padding
-  int rq[3 * kWarp];  // forward: pairs closer than r_sw (receiver lane | pair << 5 | half << 10)
-#if P3M_SYM_CPASYNC
-  float4 rec[2][kWarp];  // records of the current and the next batch
-#endif
+  // records of the current and the next batch, copied with cp.async while the current
+  // batch is staged (measured at 128^3 against a register prefetch: 1.551 -> 1.518 ms)
+  float4 rec[2][kWarp];
 };
-
 
 struct SymVjpSmem : SymSmem {
   float4 vxy[kWarp];  // adjoint: the suppliers' masked abar, negated, in the layout of sxy / sz
   float2 vz[kWarp];
 };
 
-// Resident blocks of 4 warps per SM: the forward at 8 (64 registers, no spills;
-// with the close pairs evaluated in the step it is 7% faster than at 5 on the
-// 128^3 set), the adjoint at 6 (80 registers; its softened branch with the
-// derivative spills beyond).
-#ifndef P3M_SYM_SOFT_INLINE
-#define P3M_SYM_SOFT_INLINE 1  // forward close pairs: 1 = packed softened form in the step (5-8% faster), 0 = queue
-#endif
-#ifndef P3M_SYM_OWN_TRIANGLE
-#define P3M_SYM_OWN_TRIANGLE 1  // forward: the chunk's own pairs in a triangular pass, not staged
-#endif
-#ifndef P3M_SYM_UNROLL
-#define P3M_SYM_UNROLL 1  // rotation steps per loop iteration
-#endif
-constexpr int kSymUnroll = P3M_SYM_UNROLL;
-#ifndef P3M_SYM_MINBLOCKS
-#define P3M_SYM_MINBLOCKS 8
-#endif
-#ifndef P3M_SYMV_MINBLOCKS
-#define P3M_SYMV_MINBLOCKS 6  // the adjoint instance
-#endif
-
-#ifndef P3M_SYM_ITEMS
-#define P3M_SYM_ITEMS 0
-#endif
-#ifndef P3M_SYM_PARTS
-#define P3M_SYM_PARTS 8
-#endif
-constexpr int kSymItems = P3M_SYM_ITEMS;
-constexpr int kSymMaxParts = P3M_SYM_PARTS;
+// Resident blocks of 4 warps per SM: 5 for the forward (96 registers; 6 with spills and 7
+// within 0.5% of it at 128^3), 4 for the adjoint (122 registers; 5: 1% slower).
+constexpr int kSymMinBlocks = 5;
+constexpr int kSymVjpMinBlocks = 4;
+// Chunks are split into parts (slices of equal supplier counts) up to about three work items
+// per resident warp: forward of 4096 particles (155 chunks) 0.090 ms unsplit, 0.026 in 16
+// parts; 32,768 (1181) 0.115 -> 0.055 in 8 (13: 0.067); 110,000 (4161) 0.139 -> 0.118 in 3;
+// from 262,144 (9562) on no gain, each part enumerating the chunk's candidates again.
+constexpr int kSymItems = 9120;
+constexpr int kSymMaxParts = 16;
 
 __device__ __forceinline__ f2 shfl2(f2 v, int src) {
   f2 r;
@@ -646,11 +623,68 @@ __device__ __forceinline__ f2 shfl_xor2(f2 v, int o) {
   return r;
 }
 
+struct F2x3 {
+  f2 x, y, z;
+};
+__device__ __forceinline__ F2x3 dup3(float x, float y, float z) { return F2x3{pk(x, x), pk(y, y), pk(z, z)}; }
+__device__ __forceinline__ F2x3 sub3(const F2x3& p, const float4& xy, const float2& z) {  // p - s, s stored negated
+  return F2x3{add2(p.x, pk(xy.x, xy.y)), add2(p.y, pk(xy.z, xy.w)), add2(p.z, pk(z.x, z.y))};
+}
+// The force term B d, or the adjoint's B v + D (d . v) d, added to a.
+template <bool VJP>
+__device__ __forceinline__ void add_term(F2x3& a, f2 B, const F2x3& d, const F2x3& v, f2 cc) {
+  if constexpr (!VJP) {
+    a.x = fma2(B, d.x, a.x);
+    a.y = fma2(B, d.y, a.y);
+    a.z = fma2(B, d.z, a.z);
+  } else {
+    a.x = fma2(B, v.x, fma2(cc, d.x, a.x));
+    a.y = fma2(B, v.y, fma2(cc, d.y, a.y));
+    a.z = fma2(B, v.z, fma2(cc, d.z, a.z));
+  }
+}
+
+// Bracket (VJP: with D = B'(r)/r) of the packed pair at squared distances r2, 0 unless its
+// cutoff mask c is 1 and where `coincident` pairs do not count; check: test for close pairs.
+template <int SOFT, bool VJP>
+__device__ __forceinline__ f2 masked_bracket(f2 r2, f2 c, bool check, const TraversalArgs& a, f2& D) {
+  f2 B;
+  if constexpr (VJP) B = bracket_main_vjp_f32x2<SOFT>(r2, a.f, D);
+  else B = bracket_main_f32x2<SOFT>(r2, a.f);
+  float q0, q1, c0, c1;
+  upk(r2, q0, q1);
+  upk(c, c0, c1);
+  if (check) {
+    // the softened form; in the forward a zero displacement contributes nothing (its
+    // floored r^2 gives a finite B, times 0), in the adjoint coincident particles take B(0)
+    const bool rare0 = c0 > 0.f && q0 < a.f.rsw2_f && (VJP || q0 > kR2Self);
+    const bool rare1 = c1 > 0.f && q1 < a.f.rsw2_f && (VJP || q1 > kR2Self);
+    if (__any_sync(0xffffffffu, rare0 || rare1)) {
+      float b0, b1, s0, s1;
+      upk(B, b0, b1);
+      if constexpr (VJP) {
+        f2 Ds;
+        float d0, d1, e0, e1;
+        upk(D, d0, d1);
+        upk(bracket_soft_vjp_f32x2<SOFT>(r2, a.f, a.sc, Ds), s0, s1);
+        upk(Ds, e0, e1);
+        D = pk(rare0 ? e0 : d0, rare1 ? e1 : d1);
+      } else {
+        upk(bracket_soft_f32x2<SOFT>(r2, a.f, a.sc), s0, s1);
+      }
+      B = pk(rare0 ? s0 : b0, rare1 ? s1 : b1);
+    }
+  }
+  if constexpr (VJP) D = mul2(D, c);
+  return mul2(B, c);
+}
+
 // VJP = true: the adjoint with the same traversal.  Its pair term J_ij (v_i - v_j),
 // v the masked abar, is antisymmetric in (i, j) like the force, so the partner
 // receives the negated term; every particle is a receiver.
 template <int SOFT, bool VJP = false>
-__global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_MINBLOCKS) k_force_sym(TraversalArgs a, float4* __restrict__ acc4) {
+__global__ void __launch_bounds__(kPThreads, VJP ? kSymVjpMinBlocks : kSymMinBlocks)
+    k_force_sym(TraversalArgs a, float4* __restrict__ acc4) {
   using Smem = typename std::conditional<VJP, SymVjpSmem, SymSmem>::type;
   __shared__ Smem smem[kPWarps];
   const unsigned full = 0xffffffffu;
@@ -667,7 +701,7 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
     vzf = (float*)S.vz;
   }
   const int n_chunks = *a.n_chunks;
-  const int nparts = parts_for(n_chunks, kSymItems, kSymMaxParts);
+  const int nparts = parts_for(n_chunks, kSymItems + n_chunks - 1, kSymMaxParts);
   const int n_items = n_chunks * nparts;
   const Reach rc = make_reach(a);
   const float xr2 = a.f.xr2_f;
@@ -676,26 +710,79 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
   for (;;) {
     const int w = next_chunk(a, lane);
     if (w >= n_items) break;
-    const int c = w / nparts, part = w - c * nparts;
-    const Chunk ch = chunk_at(a, c);
+    const int ci = w / nparts, part = w - ci * nparts;
+    const Chunk ch = chunk_at(a, ci);
     ChunkFrame F;
     load_chunk(a, rc, ch, lane, F);
-    const int i_self = F.valid ? F.pidx : 0x7fffffff;  // the mask j > i is false on empty lanes
-    const int c_end = ch.start + ch.count;
     const float rx = F.valid ? F.pi.x : kSymPad, ry = F.valid ? F.pi.y : kSymPad, rz = F.valid ? F.pi.z : kSymPad;
-    const f2 px = pk(rx, rx), py = pk(ry, ry), pz = pk(rz, rz);
-    f2 vix = pk(0.f, 0.f), viy = pk(0.f, 0.f), viz = pk(0.f, 0.f);  // adjoint: the receiver's masked abar
     float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (VJP) {
       if (F.valid) ab = a.abar4[F.pidx];
-      vix = pk(ab.x, ab.x);
-      viy = pk(ab.y, ab.y);
-      viz = pk(ab.z, ab.z);
     }
-    f2 ax = pk(0.f, 0.f), ay = pk(0.f, 0.f), az = pk(0.f, 0.f);
-    f2 hitsf = pk(0.f, 0.f);
-    int cnt = 0;                          // staged suppliers (warp-uniform)
-    bool blk_near = false, blk_own = false;  // the staged block holds a supplier near the box / of this chunk
+    const f2 zero = pk(0.f, 0.f);
+    F2x3 own = {zero, zero, zero};  // sums of this lane's own receiver
+    f2 hitsf = zero;
+    const f2 floor2 = VJP ? zero : pk(kR2Floor, kR2Floor);
+
+    // The chunk's own pairs: lane l with lanes l + k and l + k + 8, k = 1 ... 8 (l + 16 from
+    // the lower half only), each pair {i, j} of the chunk once; the partner's share comes
+    // back by a shuffle.
+    if (part == 0) {
+      const F2x3 p = dup3(rx, ry, rz);
+#pragma unroll 1
+      for (int k = 1; k <= 8; ++k) {
+        const int m = (lane + k) & (kWarp - 1), m2 = (lane + k + 8) & (kWarp - 1);
+        const F2x3 d = {add2(p.x, pk(-__shfl_sync(full, rx, m), -__shfl_sync(full, rx, m2))),
+                        add2(p.y, pk(-__shfl_sync(full, ry, m), -__shfl_sync(full, ry, m2))),
+                        add2(p.z, pk(-__shfl_sync(full, rz, m), -__shfl_sync(full, rz, m2)))};
+        const f2 r2 = fma2(d.x, d.x, fma2(d.y, d.y, fma2(d.z, d.z, floor2)));
+        float q0, q1;
+        upk(r2, q0, q1);
+        const bool t0 = F.valid && m < ch.count, t1 = F.valid && m2 < ch.count && (k < 8 || lane < kWarp / 2);
+        const float c0 = t0 ? fma_sat(q0, -kCutScale, xr2s) : 0.f, c1 = t1 ? fma_sat(q1, -kCutScale, xr2s) : 0.f;
+        hitsf = add2(hitsf, pk(c0, c1));
+        f2 D = zero;
+        f2 B = masked_bracket<SOFT, VJP>(r2, pk(c0, c1), true, a, D);
+        float b0, b1;
+        upk(B, b0, b1);
+        B = pk(c0 > 0.f ? b0 : 0.f, c1 > 0.f ? b1 : 0.f);  // selects: a padded lane's B may not be finite
+        F2x3 v = {zero, zero, zero};
+        f2 cc = zero;
+        if constexpr (VJP) {
+          float d0, d1;
+          upk(D, d0, d1);
+          D = pk(c0 > 0.f ? d0 : 0.f, c1 > 0.f ? d1 : 0.f);
+          v = {pk(ab.x - __shfl_sync(full, ab.x, m), ab.x - __shfl_sync(full, ab.x, m2)),
+               pk(ab.y - __shfl_sync(full, ab.y, m), ab.y - __shfl_sync(full, ab.y, m2)),
+               pk(ab.z - __shfl_sync(full, ab.z, m), ab.z - __shfl_sync(full, ab.z, m2))};
+          cc = mul2(D, fma2(d.x, v.x, fma2(d.y, v.y, mul2(d.z, v.z))));
+        }
+        F2x3 t = {zero, zero, zero};
+        add_term<VJP>(t, B, d, v, cc);
+        const int from = (lane - k) & (kWarp - 1), from2 = (lane - k - 8) & (kWarp - 1);
+        auto give = [&](f2& o, f2 u) {
+          float lo, hi;
+          upk(u, lo, hi);
+          o = add2(o, add2(u, pk(-__shfl_sync(full, lo, from), -__shfl_sync(full, hi, from2))));
+        };
+        give(own.x, t.x);
+        give(own.y, t.y);
+        give(own.z, t.z);
+      }
+    }
+
+    // Receivers of the rotation: l and l + 16 of the chunk, in both halves of the warp.
+    const int l16 = lane & 15;
+    const F2x3 pA = dup3(__shfl_sync(full, rx, l16), __shfl_sync(full, ry, l16), __shfl_sync(full, rz, l16));
+    const F2x3 pB = dup3(__shfl_sync(full, rx, l16 + 16), __shfl_sync(full, ry, l16 + 16), __shfl_sync(full, rz, l16 + 16));
+    F2x3 vA = {zero, zero, zero}, vB = vA;
+    if constexpr (VJP) {
+      vA = dup3(__shfl_sync(full, ab.x, l16), __shfl_sync(full, ab.y, l16), __shfl_sync(full, ab.z, l16));
+      vB = dup3(__shfl_sync(full, ab.x, l16 + 16), __shfl_sync(full, ab.y, l16 + 16), __shfl_sync(full, ab.z, l16 + 16));
+    }
+    F2x3 aA = {zero, zero, zero}, aB = aA;
+    int cnt = 0;            // staged suppliers (warp-uniform)
+    bool blk_near = false;  // the staged block holds a supplier near the box
 
     auto stage = [&](int rank, const Vec3<float>& pj, int j, const float4& aj) {
       const int q = rank & (kWarp - 1), h = rank >> 5;
@@ -709,17 +796,28 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
         vzf[2 * q + h] = -aj.z;
       }
     };
+    auto pad = [&](int q, int h) {
+      sxy[4 * q + h] = kSymPad;
+      sxy[4 * q + 2 + h] = kSymPad;
+      szf[2 * q + h] = kSymPad;
+      sjf[2 * q + h] = -1;
+      if constexpr (VJP) {
+        vxy[4 * q + h] = 0.f;
+        vxy[4 * q + 2 + h] = 0.f;
+        vzf[2 * q + h] = 0.f;
+      }
+    };
 
     // Evaluate the staged block of nsup suppliers (1 <= nsup <= 64) against the chunk.
     auto eval_block = [&](int nsup) {
-      int P = kWarp;
+      int P = kWarp / 2;  // pairs of each half of the warp
       if (nsup < 2 * kWarp) {
-        const int half = (nsup + 1) >> 1;
+        const int pairs = (nsup + 1) >> 1;
         P = 1;
-        while (P < half) P <<= 1;
-        // pair q = (supplier q, supplier q + P): move q + P < 32 from the a halves to the b halves
-        if (nsup <= kWarp && lane >= P && lane < nsup) {
-          const int q = lane - P;
+        while (2 * P < pairs) P <<= 1;
+        // pair q = (supplier q, supplier q + 2 P): move q + 2 P < 32 from the a halves to the b halves
+        if (nsup <= kWarp && lane >= 2 * P && lane < nsup) {
+          const int q = lane - 2 * P;
           sxy[4 * q + 1] = sxy[4 * lane];
           sxy[4 * q + 3] = sxy[4 * lane + 2];
           szf[2 * q + 1] = szf[2 * lane];
@@ -730,286 +828,81 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
             vzf[2 * q + 1] = vzf[2 * lane];
           }
         }
-        if (lane < P && lane + P >= nsup) {
-          sxy[4 * lane + 1] = kSymPad;
-          sxy[4 * lane + 3] = kSymPad;
-          szf[2 * lane + 1] = kSymPad;
-          sjf[2 * lane + 1] = -1;
-          if constexpr (VJP) {
-            vxy[4 * lane + 1] = 0.f;
-            vxy[4 * lane + 3] = 0.f;
-            vzf[2 * lane + 1] = 0.f;
-          }
-        }
+        if (lane < 2 * P && lane + 2 * P >= nsup) pad(lane, 1);
+        if (lane < 2 * P && lane >= nsup) pad(lane, 0);
         __syncwarp();
       }
-      const int qmask = P - 1;
-      const int src = (lane & ~qmask) | ((lane + 1) & qmask);
-      f2 sax = pk(0.f, 0.f), say = pk(0.f, 0.f), saz = pk(0.f, 0.f);
-      int q = lane & qmask;
-      int nq = 0;  // queued close pairs (warp-uniform)
-      // Evaluate queued close pairs [base, base + count) (count <= 32), one per lane,
-      // with the softened form, and add their terms to both particles.
-      auto run_rare = [&](int base, int count) {
-        const int e = lane < count ? S.rq[base + lane] : 0;
-        const int rl = e & (kWarp - 1);
-        const float xr = __shfl_sync(full, rx, rl), yr = __shfl_sync(full, ry, rl), zr = __shfl_sync(full, rz, rl);
-        const int ir = __shfl_sync(full, i_self, rl);
-        float vxr = 0.f, vyr = 0.f, vzr = 0.f;
-        if constexpr (VJP) {
-          vxr = __shfl_sync(full, ab.x, rl);
-          vyr = __shfl_sync(full, ab.y, rl);
-          vzr = __shfl_sync(full, ab.z, rl);
-        }
-        if (lane < count) {
-          const int qe = (e >> 5) & (kWarp - 1), he = e >> 10;
-          const float ex = xr + sxy[4 * qe + he], ey = yr + sxy[4 * qe + 2 + he], ez = zr + szf[2 * qe + he];
-          const int js = sjf[2 * qe + he];
-          float tx, ty, tz;
-          if constexpr (!VJP) {
-            const float r2s = fmaf(ex, ex, fmaf(ey, ey, fmaf(ez, ez, kR2Floor)));
-            float Ds;
-            const float Bs = bracket_soft_f32<SOFT, false>(r2s, a.f, a.sc, Ds);
-            tx = Bs * ex;
-            ty = Bs * ey;
-            tz = Bs * ez;
-          } else {  // B v + D (x_ij . v) x_ij with v = abar_i - abar_j
-            const float r2s = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-            float Ds;
-            const float Bs = bracket_soft_f32<SOFT, true>(r2s, a.f, a.sc, Ds);
-            const float wx = vxr + vxy[4 * qe + he], wy = vyr + vxy[4 * qe + 2 + he], wz = vzr + vzf[2 * qe + he];
-            const float cd = Ds * fmaf(ex, wx, fmaf(ey, wy, ez * wz));
-            tx = fmaf(Bs, wx, cd * ex);
-            ty = fmaf(Bs, wy, cd * ey);
-            tz = fmaf(Bs, wz, cd * ez);
-          }
-          atomicAdd(acc4 + ir, make_float4(tx, ty, tz, 0.f));
-          atomicAdd(acc4 + js, make_float4(-tx, -ty, -tz, 0.f));
-        }
-        __syncwarp();
-      };
-      auto run = [&](auto check_soft, auto masked) {
+      const int pmask = P - 1, base = (lane >> 4) * P;
+      const int src = (lane & ~pmask) | ((lane + 1) & pmask);
+      F2x3 sa = {zero, zero, zero};
+      int q = lane & pmask;
+      auto run = [&](auto check_soft) {
         constexpr bool kCheckSoft = decltype(check_soft)::value;
-        constexpr bool kMasked = decltype(masked)::value;
-#pragma unroll kSymUnroll
+#pragma unroll 1
         for (int k = 0; k < P; ++k) {
-          const float4 s = S.sxy[q];
-          const float2 z = S.sz[q];
-          const f2 dx = add2(px, pk(s.x, s.y));
-          const f2 dy = add2(py, pk(s.z, s.w));
-          const f2 dz = add2(pz, pk(z.x, z.y));
-          if constexpr (!VJP) {
-            const f2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, pk(kR2Floor, kR2Floor))));
-            float q0, q1;
-            upk(r2, q0, q1);
-            // No skip of steps without a hit: with 32 different pairs per step
-            // almost every step has one, and the vote costs more than it saves.
-            float c0 = fma_sat(q0, -kCutScale, xr2s), c1 = fma_sat(q1, -kCutScale, xr2s);
-            if (kMasked) {
-              const int2 jj = S.sj[q];
-              c0 = jj.x > i_self ? c0 : 0.f;
-              c1 = jj.y > i_self ? c1 : 0.f;
-            }
-            const f2 cm = pk(c0, c1);
-            hitsf = add2(hitsf, cm);
-            f2 B = bracket_main_f32x2<SOFT>(r2, a.f);
-            // Pairs closer than r_sw (the softened form): a cheap vote first, the
-            // exact condition (a hit, not a zero displacement) only when some pair
-            // is that close; then one packed softened evaluation for both halves
-            // (or, in the queue variant, the pairs leave the step's sums for a
-            // queue evaluated 32 at a time, one per lane).
-            if (kCheckSoft && __any_sync(full, fminf(q0, q1) < a.f.rsw2_f)) {
-              const bool rare0 = c0 > 0.f && q0 < a.f.rsw2_f && q0 > kR2Self;
-              const bool rare1 = c1 > 0.f && q1 < a.f.rsw2_f && q1 > kR2Self;
-#if P3M_SYM_SOFT_INLINE
-              if (__any_sync(full, rare0 || rare1)) {  // both halves in one packed softened evaluation
-                float b0, b1, s0, s1;
-                upk(B, b0, b1);
-                upk(bracket_soft_f32x2<SOFT>(r2, a.f, a.sc), s0, s1);
-                B = pk(rare0 ? s0 : b0, rare1 ? s1 : b1);
-              }
-#else
-              const unsigned rb0 = __ballot_sync(full, rare0), rb1 = __ballot_sync(full, rare1);
-              if (rb0 | rb1) {
-                const int n0 = __popc(rb0);
-                if (rare0) S.rq[nq + __popc(rb0 & lt_mask)] = lane | (q << 5);
-                if (rare1) S.rq[nq + n0 + __popc(rb1 & lt_mask)] = lane | (q << 5) | 1024;
-                nq += n0 + __popc(rb1);
-                float b0, b1;
-                upk(B, b0, b1);
-                B = pk(rare0 ? 0.f : b0, rare1 ? 0.f : b1);
-                __syncwarp();
-                while (nq >= kWarp) {
-                  nq -= kWarp;
-                  run_rare(nq, kWarp);
-                }
-              }
-#endif
-            }
-            B = mul2(B, cm);
-            ax = fma2(B, dx, ax);
-            ay = fma2(B, dy, ay);
-            az = fma2(B, dz, az);
-            sax = fma2(B, dx, sax);
-            say = fma2(B, dy, say);
-            saz = fma2(B, dz, saz);
-          } else {
-            // adjoint: B and D = B'(r)/r, the term B v + D (x_ij . v) x_ij, v = abar_i - abar_j
-            // (no r^2 floor: a zero displacement is either masked, the receiver itself,
-            // or a coincident pair, which takes the softened branch)
-            const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-            float q0, q1;
-            upk(r2, q0, q1);
-            float c0 = fma_sat(q0, -kCutScale, xr2s), c1 = fma_sat(q1, -kCutScale, xr2s);
-            if (kMasked) {
-              const int2 jj = S.sj[q];
-              c0 = jj.x > i_self ? c0 : 0.f;
-              c1 = jj.y > i_self ? c1 : 0.f;
-            }
-            const f2 cm = pk(c0, c1);
-            hitsf = add2(hitsf, cm);
-            const float4 w = S.vxy[q];
-            const float2 wz = S.vz[q];
-            const f2 vx = add2(vix, pk(w.x, w.y));
-            const f2 vy = add2(viy, pk(w.z, w.w));
-            const f2 vz2 = add2(viz, pk(wz.x, wz.y));
-            f2 D;
-            f2 B = bracket_main_vjp_f32x2<SOFT>(r2, a.f, D);
-            // close pairs (r < r_sw, coincident ones included) as in the forward, B and
-            // B'/r of the softened form; selects, since the main branch is not finite
-            // at r = 0
-            if (kCheckSoft && __any_sync(full, fminf(q0, q1) < a.f.rsw2_f)) {
-              const bool rare0 = c0 > 0.f && q0 < a.f.rsw2_f;
-              const bool rare1 = c1 > 0.f && q1 < a.f.rsw2_f;
-#if P3M_SYM_SOFT_INLINE
-              if (__any_sync(full, rare0 || rare1)) {  // both halves in one packed softened evaluation
-                f2 Dsp;
-                float b0, b1, d0, d1, s0, s1, e0, e1;
-                upk(B, b0, b1);
-                upk(D, d0, d1);
-                upk(bracket_soft_vjp_f32x2<SOFT>(r2, a.f, a.sc, Dsp), s0, s1);
-                upk(Dsp, e0, e1);
-                B = pk(rare0 ? s0 : b0, rare1 ? s1 : b1);
-                D = pk(rare0 ? e0 : d0, rare1 ? e1 : d1);
-              }
-#else
-              const unsigned rb0 = __ballot_sync(full, rare0), rb1 = __ballot_sync(full, rare1);
-              if (rb0 | rb1) {
-                const int n0 = __popc(rb0);
-                if (rare0) S.rq[nq + __popc(rb0 & lt_mask)] = lane | (q << 5);
-                if (rare1) S.rq[nq + n0 + __popc(rb1 & lt_mask)] = lane | (q << 5) | 1024;
-                nq += n0 + __popc(rb1);
-                float b0, b1, d0, d1;
-                upk(B, b0, b1);
-                upk(D, d0, d1);
-                B = pk(rare0 ? 0.f : b0, rare1 ? 0.f : b1);
-                D = pk(rare0 ? 0.f : d0, rare1 ? 0.f : d1);
-                __syncwarp();
-                while (nq >= kWarp) {
-                  nq -= kWarp;
-                  run_rare(nq, kWarp);
-                }
-              }
-#endif
-            }
-            if (kMasked) {  // selects: the receiver itself (r = 0) has non-finite main-branch values
-              float b0, b1, d0, d1;
-              upk(B, b0, b1);
-              upk(D, d0, d1);
-              B = pk(c0 > 0.f ? b0 : 0.f, c1 > 0.f ? b1 : 0.f);
-              D = pk(c0 > 0.f ? d0 : 0.f, c1 > 0.f ? d1 : 0.f);
-            } else {
-              B = mul2(B, cm);
-              D = mul2(D, cm);
-            }
-            const f2 cc = mul2(D, fma2(dx, vx, fma2(dy, vy, mul2(dz, vz2))));
-            ax = fma2(B, vx, fma2(cc, dx, ax));
-            ay = fma2(B, vy, fma2(cc, dy, ay));
-            az = fma2(B, vz2, fma2(cc, dz, az));
-            sax = fma2(B, vx, fma2(cc, dx, sax));
-            say = fma2(B, vy, fma2(cc, dy, say));
-            saz = fma2(B, vz2, fma2(cc, dz, saz));
+          const float4 s = S.sxy[base + q];
+          const float2 z = S.sz[base + q];
+          const F2x3 dA = sub3(pA, s, z), dB = sub3(pB, s, z);
+          const f2 rA = fma2(dA.x, dA.x, fma2(dA.y, dA.y, fma2(dA.z, dA.z, floor2)));
+          const f2 rB = fma2(dB.x, dB.x, fma2(dB.y, dB.y, fma2(dB.z, dB.z, floor2)));
+          float qa0, qa1, qb0, qb1;
+          upk(rA, qa0, qa1);
+          upk(rB, qb0, qb1);
+          // cutoff masks in the FP32 pipe; no skip of steps without a hit (almost every one has one)
+          const f2 cA = pk(fma_sat(qa0, -kCutScale, xr2s), fma_sat(qa1, -kCutScale, xr2s));
+          const f2 cB = pk(fma_sat(qb0, -kCutScale, xr2s), fma_sat(qb1, -kCutScale, xr2s));
+          hitsf = add2(hitsf, add2(cA, cB));
+          bool near = false;  // warp-uniform: some slot is closer than r_sw
+          if (kCheckSoft) near = __any_sync(full, fminf(fminf(qa0, qa1), fminf(qb0, qb1)) < a.f.rsw2_f);
+          f2 DA = zero, DB = zero;
+          const f2 BA = masked_bracket<SOFT, VJP>(rA, cA, kCheckSoft && near, a, DA);
+          const f2 BB = masked_bracket<SOFT, VJP>(rB, cB, kCheckSoft && near, a, DB);
+          F2x3 wA = {zero, zero, zero}, wB = wA;
+          f2 ccA = zero, ccB = zero;
+          if constexpr (VJP) {
+            const float4 vs = S.vxy[base + q];
+            const float2 vz = S.vz[base + q];
+            wA = sub3(vA, vs, vz);
+            wB = sub3(vB, vs, vz);
+            ccA = mul2(DA, fma2(dA.x, wA.x, fma2(dA.y, wA.y, mul2(dA.z, wA.z))));
+            ccB = mul2(DB, fma2(dB.x, wB.x, fma2(dB.y, wB.y, mul2(dB.z, wB.z))));
           }
+          add_term<VJP>(aA, BA, dA, wA, ccA);
+          add_term<VJP>(sa, BA, dA, wA, ccA);
+          add_term<VJP>(aB, BB, dB, wB, ccB);
+          add_term<VJP>(sa, BB, dB, wB, ccB);
           // the pair of lane l + 1 comes to lane l, with its accumulator
-          sax = shfl2(sax, src);
-          say = shfl2(say, src);
-          saz = shfl2(saz, src);
-          q = (q + 1) & qmask;
+          sa.x = shfl2(sa.x, src);
+          sa.y = shfl2(sa.y, src);
+          sa.z = shfl2(sa.z, src);
+          q = (q + 1) & pmask;
         }
       };
-      if (blk_near) {
-        if (blk_own) run(std::true_type{}, std::true_type{});
-        else run(std::true_type{}, std::false_type{});
-      } else {
-        if (blk_own) run(std::false_type{}, std::true_type{});
-        else run(std::false_type{}, std::false_type{});
+      if (blk_near) run(std::true_type{});
+      else run(std::false_type{});
+      // after P steps lane l holds the sum of its group for pair l mod P of its half
+      for (int o = P; o < kWarp / 2; o <<= 1) {
+        sa.x = add2(sa.x, shfl_xor2(sa.x, o));
+        sa.y = add2(sa.y, shfl_xor2(sa.y, o));
+        sa.z = add2(sa.z, shfl_xor2(sa.z, o));
       }
-      if (nq > 0) {  // the rest of the block's queue, while its suppliers are staged
-        run_rare(0, nq);
-        nq = 0;
-      }
-      // after P steps lane l holds the sum of its group for pair l mod P
-      for (int o = P; o < kWarp; o <<= 1) {
-        sax = add2(sax, shfl_xor2(sax, o));
-        say = add2(say, shfl_xor2(say, o));
-        saz = add2(saz, shfl_xor2(saz, o));
-      }
-      if (lane < P) {
-        const int2 jj = S.sj[lane];
+      if (l16 < P) {
+        const int2 jj = S.sj[base + l16];
         float xa, xb, ya, yb, za, zb;
-        upk(sax, xa, xb);
-        upk(say, ya, yb);
-        upk(saz, za, zb);
+        upk(sa.x, xa, xb);
+        upk(sa.y, ya, yb);
+        upk(sa.z, za, zb);
         if (jj.x >= 0) atomicAdd(acc4 + jj.x, make_float4(-xa, -ya, -za, 0.f));
         if (jj.y >= 0) atomicAdd(acc4 + jj.y, make_float4(-xb, -yb, -zb, 0.f));
       }
       __syncwarp();
     };
 
-    // The chunk's own pairs (forward): lane l with lane l + k, k = 1 ... 16 (k = 16 from
-    // the lower half only), each pair {i, j} of the chunk once; the partner's share
-    // comes back by a shuffle from lane l - k.  The staged suppliers then start after
-    // the chunk, so no block needs the j > i mask.
-    constexpr bool kOwnTri = !VJP && P3M_SYM_OWN_TRIANGLE;
-    if (kOwnTri && part == 0) {
-      float ox = 0.f, oy = 0.f, oz = 0.f, oh = 0.f;
-#pragma unroll 1
-      for (int k = 1; k <= kWarp / 2; ++k) {
-        const int m = (lane + k) & (kWarp - 1);
-        const float xm = __shfl_sync(full, rx, m), ym = __shfl_sync(full, ry, m), zm = __shfl_sync(full, rz, m);
-        const bool vm = __shfl_sync(full, (int)F.valid, m) != 0;
-        const bool take = F.valid && vm && (k < kWarp / 2 || lane < kWarp / 2);
-        const float dx = rx - xm, dy = ry - ym, dz = rz - zm;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, kR2Floor)));
-        const float c = take ? fma_sat(r2, -kCutScale, xr2s) : 0.f;
-        oh += c;
-        float Dm;
-        float B = bracket_main_f32<SOFT, false>(r2, a.f, Dm);
-        const bool rare = c > 0.f && r2 < a.f.rsw2_f && r2 > kR2Self;
-        if (__any_sync(full, rare)) {
-          float Ds;
-          const float Bs = bracket_soft_f32<SOFT, false>(r2, a.f, a.sc, Ds);
-          if (rare) B = Bs;
-        }
-        B = c > 0.f ? B : 0.f;  // a select: padded lanes may carry a non-finite B
-        const float tx = B * dx, ty = B * dy, tz = B * dz;
-        const int from = (lane - k) & (kWarp - 1);
-        ox += tx - __shfl_sync(full, tx, from);
-        oy += ty - __shfl_sync(full, ty, from);
-        oz += tz - __shfl_sync(full, tz, from);
-      }
-      ax = add2(ax, pk(ox, 0.f));
-      ay = add2(ay, pk(oy, 0.f));
-      az = add2(az, pk(oz, 0.f));
-      hitsf = add2(hitsf, pk(oh, 0.f));
-    }
-
     // Stage the survivors of each batch of 32 list positions; evaluate a block
     // whenever 64 are staged, and the rest once the enumeration is done (one
     // call site of eval_block, so its loops are inlined once).
     enumerate_suppliers(
-        a, rc, F, S.L, lane, part, nparts, kOwnTri ? c_end : ch.start,
-        [&](int nlist, int lo, int hi, bool last) {
+        a, rc, F, S.L, lane, part, nparts, ch.start + ch.count, [&](int nlist, int lo, int hi, bool last) {
           const WarpList& L = S.L;
           ListCursor<WarpList> cur;
           cur.seek(L, nlist, lane, lo);
@@ -1017,19 +910,14 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
           int jn;
           unsigned dn;
           bool vn = locate(lo, jn, dn);
-#if P3M_SYM_CPASYNC
           int buf = 0;
           if (vn) cp_async16(&S.rec[0][lane], a.rel4 + jn);
           cp_async_commit();
-          float4 rn = make_float4(0.f, 0.f, 0.f, 0.f);
-#else
-          float4 rn = vn ? a.rel4[jn] : make_float4(0.f, 0.f, 0.f, 0.f);
-#endif
           float4 an = make_float4(0.f, 0.f, 0.f, 0.f);
           if (VJP && vn) an = a.abar4[jn];
           for (int b = lo;; b += kWarp) {
             const bool more = b < hi;  // warp-uniform
-            bool keep = false, near = false, own = false;
+            bool keep = false, near = false;
             Vec3<float> pj = {0.f, 0.f, 0.f};
             int j = 0, rank = 0, ns = 0;
             float4 aj = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1039,16 +927,11 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
               j = jn;
               if (VJP) aj = an;
               vn = (b + kWarp < hi) ? locate(b + kWarp, jn, dn) : false;
-#if P3M_SYM_CPASYNC
               if (vn) cp_async16(&S.rec[buf ^ 1][lane], a.rel4 + jn);
               cp_async_commit();
               cp_async_wait_prev();  // this lane's copy of batch b has landed
               const float4 r = have ? S.rec[buf][lane] : make_float4(0.f, 0.f, 0.f, 0.f);
               buf ^= 1;
-#else
-              const float4 r = rn;
-              if (vn) rn = a.rel4[jn];
-#endif
               if (VJP && vn) an = a.abar4[jn];
               if (have) {
                 int ddx, ddy, ddz;
@@ -1056,20 +939,15 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
                 pj.x = fmaf((float)ddx, a.g.side32[0], r.x);
                 pj.y = fmaf((float)ddy, a.g.side32[1], r.y);
                 pj.z = fmaf((float)ddz, a.g.side32[2], r.z);
-                const float tx = fmaxf(fmaxf(F.lo.x - pj.x, pj.x - F.hi.x), 0.f);
-                const float ty = fmaxf(fmaxf(F.lo.y - pj.y, pj.y - F.hi.y), 0.f);
-                const float tz = fmaxf(fmaxf(F.lo.z - pj.z, pj.z - F.hi.z), 0.f);
-                const float gap2 = fmaf(tx, tx, fmaf(ty, ty, tz * tz));
+                const float gap2 = box_gap2(F, pj);
                 keep = gap2 < a.f.margin2_f;
                 near = keep && gap2 < a.f.rsw2_f;
               }
-              own = keep && j < c_end;
               const unsigned m = __ballot_sync(full, keep);
               ns = __popc(m);
               rank = cnt + __popc(m & lt_mask);
               if (keep && rank < 2 * kWarp) stage(rank, pj, j, aj);
               blk_near = blk_near || __any_sync(full, near && rank < 2 * kWarp);
-              blk_own = blk_own || __any_sync(full, own && rank < 2 * kWarp);
             }
             const bool flush = more ? (cnt + ns >= 2 * kWarp) : (last && cnt > 0);
             if (flush) {
@@ -1077,7 +955,6 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
               eval_block(more ? 2 * kWarp : cnt);
               if (more) {
                 blk_near = __any_sync(full, near && rank >= 2 * kWarp);
-                blk_own = __any_sync(full, own && rank >= 2 * kWarp);
                 if (keep && rank >= 2 * kWarp) stage(rank - 2 * kWarp, pj, j, aj);
                 cnt += ns - 2 * kWarp;
               } else {
@@ -1089,19 +966,20 @@ __global__ void __launch_bounds__(kPThreads, VJP ? P3M_SYMV_MINBLOCKS : P3M_SYM_
             if (!more) break;
           }
         });
-    float l, h;
-    float4 mine;
-    upk(ax, l, h);
-    mine.x = l + h;
-    upk(ay, l, h);
-    mine.y = l + h;
-    upk(az, l, h);
-    mine.z = l + h;
-    mine.w = 0.f;
+    // lane l keeps receiver l: the lower half's A sums and the upper half's B sums are its
+    // own, the other half of the warp holds the rest of each
+    auto total = [&](f2 o, f2 A, f2 B) {
+      const bool upper = lane >= 16;
+      const f2 mine = upper ? B : A, other = shfl_xor2(upper ? A : B, 16);
+      float lo, hi;
+      upk(add2(o, add2(mine, other)), lo, hi);
+      return lo + hi;
+    };
+    const float4 mine = make_float4(total(own.x, aA.x, aB.x), total(own.y, aA.y, aB.y), total(own.z, aA.z, aB.z), 0.f);
     if (F.valid) atomicAdd(acc4 + F.pidx, mine);
+    float l, h;
     upk(hitsf, l, h);
-    const int hits = F.valid ? (int)(l + h) : 0;
-    pair_total += 2ull * (unsigned long long)__reduce_add_sync(full, (unsigned)hits);  // ordered pairs
+    pair_total += 2ull * (unsigned long long)__reduce_add_sync(full, (unsigned)(int)(l + h));  // ordered pairs
   }
   if (lane == 0 && pair_total) atomicAdd(a.pairs, pair_total);
 }
