@@ -140,6 +140,37 @@ __device__ __forceinline__ void rel_to_subtile(const Geometry& g, double x, doub
   r[2] = __dsub_rn(z, __ldg(g.org + g.M[0] + g.M[1] + gz));
 }
 
+// float -> double and double -> float (round to nearest) on the integer pipe: the conversion
+// instructions run on the FP64 pipe, at a warp instruction in 16 clocks, and cost a pass
+// over the particles as much as its arithmetic (each conversion per particle: 3.3 us at
+// 128^3, also where it is predicated off, so there is no conversion for the rare cases in
+// line).  A subnormal float is scaled by 2^64 first; narrow leaves results that are not
+// normal floats, zero apart, to a call.
+__device__ __forceinline__ double widen(float x) {
+  const bool small = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;
+  const unsigned b = __float_as_uint(small ? x * 0x1p64f : x), m = b & 0x7fffffffu;
+  unsigned hi = (m >> 3) + (small ? 0x34000000u : 0x38000000u);
+  hi = m == 0 ? 0u : (m >= 0x7f800000u ? hi | 0x7ff00000u : hi);
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+static __device__ __noinline__ float narrow_slow(double x) { return (float)x; }
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned h = (hi & 0x7fffffffu) - 0x38000000u;       // exponent rebiased
+  const unsigned r = lo + 0x0fffffffu + ((lo >> 29) & 1u);  // to nearest, ties to even, at bit 29
+  if (h - 0x00100000u < 0x0fe00000u)
+    return __uint_as_float((hi & 0x80000000u) | __funnelshift_l(r, h + (r < lo ? 1u : 0u), 3));
+  return ((hi & 0x7fffffffu) | lo) == 0 ? __uint_as_float(hi) : narrow_slow(x);
+}
+// |x| in FP32 from the high word: less than 2^-20 below it, at least 2^-126 unless that word
+// is 0, at most 3.4e38 (infinities and NaN too).  For bounds with a margin.
+__device__ __forceinline__ float magnitude(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return h == 0 ? 0.0f : __uint_as_float((min(max(h, 0x38100000u), 0x47efffffu) - 0x38000000u) << 3);
+}
+__device__ __forceinline__ float magnitude(float x) { return fabsf(x); }
+
 // Subtile origins i * side64[d] for the table g.org (M[0] + M[1] + M[2] entries).
 __global__ void k_fill_origins(Geometry g, double* __restrict__ org);
 

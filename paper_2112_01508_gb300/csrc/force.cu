@@ -72,7 +72,7 @@ __global__ void k_rel4(const double* __restrict__ pos, const int* __restrict__ c
   }
   double r[3];
   rel_to_subtile(g, x, y, z, gx, gy, gz, r);
-  float f[3] = {(float)r[0], (float)r[1], (float)r[2]};
+  float f[3] = {narrow(r[0]), narrow(r[1]), narrow(r[2])};
   // relative to the origin of the subtile of the last sort; a particle that drifted
   // across the periodic boundary since then takes its nearest image.  Its offset is
   // then near +-L, every other one far below L/2, so the test is made in FP32, and

@@ -257,7 +257,7 @@ __global__ void k_gather_pos_rel4(const double* __restrict__ src, const int* __r
   decode_subtile(g, id, gx, gy, gz);
   double r[3];
   rel_to_subtile(g, x, y, z, gx, gy, gz, r);
-  rel4[k] = make_float4((float)r[0], (float)r[1], (float)r[2], __int_as_float(id));
+  rel4[k] = make_float4(narrow(r[0]), narrow(r[1]), narrow(r[2]), __int_as_float(id));
 }
 
 // Carried arrays of an out-of-place sort: element bytes as `words` words of
@@ -295,7 +295,7 @@ __global__ void k_gather_all(const double* __restrict__ src, const int* __restri
   decode_subtile(g, id, gx, gy, gz);
   double r[3];
   rel_to_subtile(g, x, y, z, gx, gy, gz, r);
-  rel4[k] = make_float4((float)r[0], (float)r[1], (float)r[2], __int_as_float(id));
+  rel4[k] = make_float4(narrow(r[0]), narrow(r[1]), narrow(r[2]), __int_as_float(id));
   for (int c = 0; c < cs.count; ++c) {
     switch (cs.wbytes[c]) {
       case 8: copy_words<unsigned long long>(cs.src[c], cs.dst[c], j, k, cs.words[c]); break;

@@ -1,8 +1,16 @@
 // Rung assignment (Section 2.2.2, Eq. rung), kick and drift (Section 2.2.2,
 // operators K and D with a static scale factor a = 1).  All three are
-// elementwise and HBM-bound; the arithmetic is IEEE double with explicit
-// round-to-nearest intrinsics so that the integer rung decision and the
-// updated momenta/positions are reproducible bit for bit.
+// elementwise; the arithmetic is IEEE double with explicit round-to-nearest
+// intrinsics so that the integer rung decision and the updated momenta/positions
+// are reproducible bit for bit.
+//
+// Their bound is HBM, once the FP64 pipe is spared: it retires a warp instruction in 16
+// clocks (3.3 us per instruction and particle at 128^3), conversions included.  So
+// conversions run on the integer pipe (common.cuh), FP32 kicks decide their rounding in
+// FP32 (kick_value), and all loads of a particle are in flight before the first use.  At
+// 128^3, with FP32 (FP64) momenta and FP32 accelerations: kick 66 -> 19 (46 -> 31) us,
+// drift 52 -> 33 (52 -> 33) us, kick + drift with rungs in one pass 112 -> 40 (89 -> 62) us,
+// rung kick + drift 133 -> 48 (110 -> 72) us.
 #include <algorithm>
 #include <cmath>
 
@@ -74,27 +82,106 @@ __global__ void k_rungs(const A* __restrict__ acc, int64_t n, double qq, float q
   rung[i] = (int8_t)rung_rule<A>(acc[i], acc[n + i], acc[2 * n + i], qq, qqf, n_rung, err);
 }
 
+// Kick factors K, and each as an unevaluated sum of two floats (kh = NaN where that does not
+// hold K to 2^-48, which sends FP32 kicks to FP64).
+constexpr int kMaxFactors = 24;
 struct KickFactors {
-  double k[8];
+  double k[kMaxFactors];
+  float kh[kMaxFactors], kl[kMaxFactors];
 };
+static void set_factor(KickFactors& kf, int i, double K) {
+  const double m = std::fabs(K);
+  const bool ok = m >= 0x1p-60 && m <= 0x1p60;
+  kf.k[i] = K;
+  kf.kh[i] = ok ? (float)K : std::nanf("");
+  kf.kl[i] = ok ? (float)(K - (double)(float)K) : 0.0f;
+}
+
+static __device__ __noinline__ float kick_f32_slow(float q, float a, double K) {
+  return (float)__dadd_rn((double)q, __dmul_rn((double)a, K));
+}
+
+// The kick q + a K in IEEE double, rounded once to M.
+//
+// For FP32 momenta and accelerations the FP64 pipe does not see it: a K is formed as p + e
+// from K = kh + kl, q + p as s + t exactly (Knuth's two-sum), and s + (t + e) is off the
+// exact sum by less than 2^-45 (|q| + |p|); the double result is within 2^-52 of it.  If
+// adding and subtracting 2^-42 (|q| + |p|) round to the same float, so does everything
+// between, the double result included (Ziv's rounding test); otherwise (one component in
+// about 2^17), near zero and outside the range where e is exact, the doubles decide.
+template <class M, class A>
+__device__ __forceinline__ M kick_value(M q, A a, const KickFactors& kf, int i) {
+  if constexpr (std::is_same<M, float>::value && std::is_same<A, float>::value) {
+    const float kh = kf.kh[i];
+    const float p = __fmul_rn(a, kh);
+    const float e = __fmaf_rn(a, kf.kl[i], __fmaf_rn(a, kh, -p));
+    const float s = __fadd_rn(q, p), bb = __fsub_rn(s, q);
+    const float t = __fadd_rn(__fsub_rn(q, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    const float r = __fadd_rn(t, e);
+    const float mag = __fadd_rn(fabsf(q), fabsf(p));
+    const float tol = __fmul_rn(mag, 0x1p-42f);
+    const float up = __fadd_rn(s, __fadd_rn(r, tol)), dn = __fadd_rn(s, __fsub_rn(r, tol));
+    const bool ok = up == dn && up != 0.0f && mag >= 0x1p-70f && mag <= 0x1p120f && (fabsf(p) >= 0x1p-70f || a == 0.0f);
+    return ok ? up : kick_f32_slow(q, a, kf.k[i]);
+  } else {
+    const double v = __dadd_rn(widen(q), __dmul_rn(widen(a), kf.k[i]));
+    if constexpr (std::is_same<M, float>::value) return narrow(v);
+    else return v;
+  }
+}
+
+// One coordinate of the drift: x + q factor in IEEE double, wrapped into [0, box).
+__device__ __forceinline__ double drift_value(double x, double q, double factor, double box) {
+  double v = __dadd_rn(x, __dmul_rn(q, factor));
+  const long long vb = __double_as_longlong(v);
+  if (!(vb >= 0 && vb < __double_as_longlong(box))) {  // v - L floor(v / L); floor is 0 inside the box
+    v = __dsub_rn(v, __dmul_rn(box, floor(__ddiv_rn(v, box))));
+    if (v >= box || v < 0.0) v = 0.0;
+  }
+  return v;
+}
+
+// Upper bound of the displacement |q| |factor| (FP32 with a relative margin far above its
+// rounding and the truncation of q; saturates for non-finite or huge momenta).
+__device__ __forceinline__ float disp_bound(float q2, double factor) {
+  const float d = sqrtf(q2) * (float)fabs(factor) * 1.0001f;
+  return d < 3.0e38f ? d : 3.0e38f;
+}
+
+// The drift of particle i from x with momentum q; returns its displacement bound.
+template <class M>
+__device__ __forceinline__ float drift_one(double* __restrict__ pos, const M (&q)[3], const double (&x)[3], int64_t n,
+                                           int64_t i, double factor, double box) {
+  float q2 = 0.0f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float m = magnitude(q[d]);
+    q2 = fmaf(m, m, q2);
+    pos[d * n + i] = drift_value(x[d], widen(q[d]), factor, box);
+  }
+  return disp_bound(q2, factor);
+}
 
 template <class M, class A>
 __global__ void k_kick(M* __restrict__ mom, const A* __restrict__ acc, const int8_t* __restrict__ rung, int rung_min,
-                       int64_t n, KickFactors kf) {
+                       int64_t n, const __grid_constant__ KickFactors kf) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  double k = kf.k[0];
+  int k = 0;
   if (rung) {
-    int l = rung[i];
+    const int l = rung[i];
     if (l < rung_min) return;
-    k = kf.k[l < 0 ? 0 : (l > 7 ? 7 : l)];
+    k = l < 0 ? 0 : (l > 7 ? 7 : l);
+  }
+  M q[3];
+  A av[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {  // all loads in flight before the first use
+    q[d] = mom[d * n + i];
+    av[d] = acc[d * n + i];
   }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    double q = (double)mom[d * n + i];
-    double v = __dadd_rn(q, __dmul_rn((double)acc[d * n + i], k));
-    mom[d * n + i] = (M)v;
-  }
+  for (int d = 0; d < 3; ++d) mom[d * n + i] = kick_value<M, A>(q[d], av[d], kf, k);
 }
 
 // disp (optional): receives, by atomic max, an upper bound of the largest
@@ -106,24 +193,14 @@ __global__ void __launch_bounds__(256, kKdMinBlocks) k_drift(double* __restrict_
   __shared__ unsigned warp_max[8];
   float my = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float q2 = 0.0f;
+    M q[3];
+    double x[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double q = (double)mom[d * n + i];
-      const float qf = (float)q;
-      q2 = fmaf(qf, qf, q2);
-      double v = __dadd_rn(pos[d * n + i], __dmul_rn(q, factor));
-      const long long vb = __double_as_longlong(v);
-      if (!(vb >= 0 && vb < __double_as_longlong(box))) {  // v - L floor(v / L); floor is 0 inside the box
-        v = __dsub_rn(v, __dmul_rn(box, floor(__ddiv_rn(v, box))));
-        if (v >= box || v < 0.0) v = 0.0;
-      }
-      pos[d * n + i] = v;
+      q[d] = mom[d * n + i];
+      x[d] = pos[d * n + i];
     }
-    // FP32 with a relative margin far above its rounding (a few ulps)
-    float di = sqrtf(q2) * (float)fabs(factor) * 1.0001f;
-    if (!(di < 3.0e38f)) di = 3.0e38f;  // non-finite or huge momenta: the bound saturates
-    my = fmaxf(my, di);
+    my = fmaxf(my, drift_one<M>(pos, q, x, n, i, factor, box));
   }
   if (disp) {
     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(my));
@@ -143,34 +220,28 @@ __global__ void __launch_bounds__(256, kKdMinBlocks) k_drift(double* __restrict_
 template <class M, class A>
 __global__ void __launch_bounds__(256, kKdMinBlocks) k_kick_drift(double* __restrict__ pos, M* __restrict__ mom,
                                                     const A* __restrict__ acc, int8_t* __restrict__ rung, int64_t n,
-                                                    double qq, float qqf, int n_rung, KickFactors kf, double factor,
+                                                    double qq, float qqf, int n_rung,
+                                                    const __grid_constant__ KickFactors kf, double factor,
                                                     double box, float* __restrict__ disp, int* __restrict__ err) {
   __shared__ unsigned warp_max[8];
   float my = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const A av[3] = {acc[i], acc[n + i], acc[2 * n + i]};
-    const int l = rung_rule<A>(av[0], av[1], av[2], qq, qqf, n_rung, err);
-    rung[i] = (int8_t)l;
-    const double k = kf.k[l];
-    float q2 = 0.0f;
+    M q[3];
+    double x[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const M qm = (M)__dadd_rn((double)mom[d * n + i], __dmul_rn((double)av[d], k));
-      mom[d * n + i] = qm;
-      const double q = (double)qm;
-      const float qf = (float)q;
-      q2 = fmaf(qf, qf, q2);
-      double v = __dadd_rn(pos[d * n + i], __dmul_rn(q, factor));
-      const long long vb = __double_as_longlong(v);
-      if (!(vb >= 0 && vb < __double_as_longlong(box))) {
-        v = __dsub_rn(v, __dmul_rn(box, floor(__ddiv_rn(v, box))));
-        if (v >= box || v < 0.0) v = 0.0;
-      }
-      pos[d * n + i] = v;
+      q[d] = mom[d * n + i];
+      x[d] = pos[d * n + i];
     }
-    float di = sqrtf(q2) * (float)fabs(factor) * 1.0001f;
-    if (!(di < 3.0e38f)) di = 3.0e38f;
-    my = fmaxf(my, di);
+    const int l = rung_rule<A>(av[0], av[1], av[2], qq, qqf, n_rung, err);
+    rung[i] = (int8_t)l;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      q[d] = kick_value<M, A>(q[d], av[d], kf, l);
+      mom[d * n + i] = q[d];
+    }
+    my = fmaxf(my, drift_one<M>(pos, q, x, n, i, factor, box));
   }
   if (disp) {
     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(my));
@@ -186,26 +257,27 @@ __global__ void __launch_bounds__(256, kKdMinBlocks) k_kick_drift(double* __rest
 
 // One kick of the rung-based leapfrog with the rung update (see p3m_sr_rung_kick) for
 // particle i.
+// (q: its momentum, in and out; written back if kicked)
 template <class M, class A>
-__device__ __forceinline__ void rung_kick_one(M* __restrict__ mom, const A* __restrict__ acc, int8_t* __restrict__ rung,
-                                              int8_t* __restrict__ state, int64_t n, int64_t i, int rung_min,
-                                              long long k, int log2_sub, double dt, double qq, float qqf, int n_rung,
-                                              int sync, int* __restrict__ err) {
+__device__ __forceinline__ void rung_kick_one(M* __restrict__ mom, M (&q)[3], const A* __restrict__ acc,
+                                              int8_t* __restrict__ rung, int8_t* __restrict__ state, int64_t n,
+                                              int64_t i, int rung_min, long long k, int log2_sub,
+                                              const KickFactors& kf, double qq, float qqf, int n_rung, int sync,
+                                              int* __restrict__ err) {
   const int l = rung[i];
   if (l < rung_min) return;
+  A av[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) av[d] = acc[d * n + i];
   const int st = state[i];
   if (l >= n_rung || st < 0 || st > 2) {  // corrupted rung or state: leave the particle alone
     atomicOr(err, kErrRungState);
     return;
   }
-  const double f = st == 0 ? 1.0 : (st == 1 ? 0.5 : 0.75);
-  const double fac = sync ? f - 0.5 : f;
-  const double K = ldexp(__dmul_rn(dt, fac), -l);  // fac dt / 2^l (the scaling is exact)
-  A av[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    av[d] = acc[d * n + i];
-    mom[d * n + i] = (M)__dadd_rn((double)mom[d * n + i], __dmul_rn((double)av[d], K));
+    q[d] = kick_value<M, A>(q[d], av[d], kf, st * 8 + l);
+    mom[d * n + i] = q[d];
   }
   if (sync) {
     state[i] = 0;
@@ -227,11 +299,13 @@ __device__ __forceinline__ void rung_kick_one(M* __restrict__ mom, const A* __re
 
 template <class M, class A>
 __global__ void k_rung_kick(M* __restrict__ mom, const A* __restrict__ acc, int8_t* __restrict__ rung,
-                            int8_t* __restrict__ state, int64_t n, int rung_min, long long k, int log2_sub, double dt,
-                            double qq, float qqf, int n_rung, int sync, int* __restrict__ err) {
+                            int8_t* __restrict__ state, int64_t n, int rung_min, long long k, int log2_sub,
+                            const __grid_constant__ KickFactors kf, double qq, float qqf, int n_rung, int sync,
+                            int* __restrict__ err) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  rung_kick_one<M, A>(mom, acc, rung, state, n, i, rung_min, k, log2_sub, dt, qq, qqf, n_rung, sync, err);
+  M q[3] = {mom[i], mom[n + i], mom[2 * n + i]};
+  rung_kick_one<M, A>(mom, q, acc, rung, state, n, i, rung_min, k, log2_sub, kf, qq, qqf, n_rung, sync, err);
 }
 
 // A rung kick followed by the drift of every particle, in one pass (the results of
@@ -239,31 +313,23 @@ __global__ void k_rung_kick(M* __restrict__ mom, const A* __restrict__ acc, int8
 template <class M, class A>
 __global__ void __launch_bounds__(256, kKdMinBlocks) k_rung_kick_drift(M* __restrict__ mom, const A* __restrict__ acc,
                                                          int8_t* __restrict__ rung, int8_t* __restrict__ state,
-                                                         int64_t n, int rung_min, long long k, int log2_sub, double dt,
+                                                         int64_t n, int rung_min, long long k, int log2_sub,
+                                                         const __grid_constant__ KickFactors kf,
                                                          double qq, float qqf, int n_rung, int* __restrict__ err,
                                                          double* __restrict__ pos, double factor, double box,
                                                          float* __restrict__ disp) {
   __shared__ unsigned warp_max[8];
   float my = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    rung_kick_one<M, A>(mom, acc, rung, state, n, i, rung_min, k, log2_sub, dt, qq, qqf, n_rung, 0, err);
-    float q2 = 0.0f;
+    M q[3];
+    double x[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double q = (double)mom[d * n + i];
-      const float qf = (float)q;
-      q2 = fmaf(qf, qf, q2);
-      double v = __dadd_rn(pos[d * n + i], __dmul_rn(q, factor));
-      const long long vb = __double_as_longlong(v);
-      if (!(vb >= 0 && vb < __double_as_longlong(box))) {
-        v = __dsub_rn(v, __dmul_rn(box, floor(__ddiv_rn(v, box))));
-        if (v >= box || v < 0.0) v = 0.0;
-      }
-      pos[d * n + i] = v;
+      q[d] = mom[d * n + i];
+      x[d] = pos[d * n + i];
     }
-    float di = sqrtf(q2) * (float)fabs(factor) * 1.0001f;
-    if (!(di < 3.0e38f)) di = 3.0e38f;
-    my = fmaxf(my, di);
+    rung_kick_one<M, A>(mom, q, acc, rung, state, n, i, rung_min, k, log2_sub, kf, qq, qqf, n_rung, 0, err);
+    my = fmaxf(my, drift_one<M>(pos, q, x, n, i, factor, box));
   }
   if (disp) {
     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(my));
@@ -325,7 +391,7 @@ extern "C" p3m_status p3m_sr_kick_drift(p3m_sr_ctx* ctx, double* pos, void* mom,
   if (ctx->n == 0) return P3M_OK;
   const double qq = rung_qq(dt, eta, eps);
   KickFactors kf{};
-  for (int l = 0; l < ctx->prm.n_rung; ++l) kf.k[l] = kick_factor[l];
+  for (int l = 0; l < ctx->prm.n_rung; ++l) set_factor(kf, l, kick_factor[l]);
   float* slot = drift_slot(ctx, pos);
   const int t = 256;
   const int64_t n = ctx->n;
@@ -394,7 +460,7 @@ extern "C" p3m_status p3m_sr_kick(p3m_sr_ctx* ctx, void* mom, int mom_precision,
   if (st != P3M_OK) return st;
   if (ctx->n == 0) return P3M_OK;
   KickFactors kf{};
-  for (int l = 0; l < ctx->prm.n_rung; ++l) kf.k[l] = kick_factor[l];
+  for (int l = 0; l < ctx->prm.n_rung; ++l) set_factor(kf, l, kick_factor[l]);
   const int t = 256;
   const unsigned b = blocks_for(ctx->n, t);
   cudaStream_t s = ctx->stream;
@@ -420,7 +486,7 @@ extern "C" p3m_status p3m_sr_drift(p3m_sr_ctx* ctx, double* pos, const void* mom
   if (ctx->n == 0) return P3M_OK;
   float* slot = drift_slot(ctx, pos);
   const int t = 256;
-  const unsigned b = blocks_for(ctx->n, t);
+  const unsigned b = (unsigned)std::min<int64_t>(blocks_for(ctx->n, t), (int64_t)ctx->num_sms * 8);
   if (mom_precision == 64)
     { k_drift<double><<<b, t, 0, ctx->stream>>>(pos, (const double*)mom, ctx->n, factor, ctx->prm.box, slot);
       ++ctx->launches; }
@@ -476,6 +542,12 @@ static p3m_status rung_kick_impl(p3m_sr_ctx* ctx, void* mom, int mom_precision, 
   volatile double t3 = t2 * eps;
   volatile double q = t1 / t3;
   const double qq = q * q;
+  KickFactors kf{};  // f dt / 2^l (the scaling is exact) by kick state and rung
+  for (int st3 = 0; st3 < 3; ++st3) {
+    const double f = st3 == 0 ? 1.0 : (st3 == 1 ? 0.5 : 0.75);
+    const double fac = synchronize ? f - 0.5 : f;
+    for (int l = 0; l < 8; ++l) set_factor(kf, st3 * 8 + l, std::ldexp(dt * fac, -l));
+  }
   const int t = 256;
   const unsigned b = blocks_for(ctx->n, t);
   cudaStream_t s = ctx->stream;
@@ -489,19 +561,19 @@ static p3m_status rung_kick_impl(p3m_sr_ctx* ctx, void* mom, int mom_precision, 
     const double L = ctx->prm.box;
     if (mom_precision == 64 && acc_precision == 32)
       k_rung_kick_drift<double, float><<<bd, t, 0, s>>>((double*)mom, (const float*)acc, rung, kick_state, n, rung_min,
-                                                        substep, log2_sub, dt, qq, qqf, nr, ctx->err_dev, pos,
+                                                        substep, log2_sub, kf, qq, qqf, nr, ctx->err_dev, pos,
                                                         drift_factor, L, slot);
     else if (mom_precision == 64 && acc_precision == 64)
       k_rung_kick_drift<double, double><<<bd, t, 0, s>>>((double*)mom, (const double*)acc, rung, kick_state, n,
-                                                         rung_min, substep, log2_sub, dt, qq, qqf, nr, ctx->err_dev,
+                                                         rung_min, substep, log2_sub, kf, qq, qqf, nr, ctx->err_dev,
                                                          pos, drift_factor, L, slot);
     else if (mom_precision == 32 && acc_precision == 32)
       k_rung_kick_drift<float, float><<<bd, t, 0, s>>>((float*)mom, (const float*)acc, rung, kick_state, n, rung_min,
-                                                       substep, log2_sub, dt, qq, qqf, nr, ctx->err_dev, pos,
+                                                       substep, log2_sub, kf, qq, qqf, nr, ctx->err_dev, pos,
                                                        drift_factor, L, slot);
     else
       k_rung_kick_drift<float, double><<<bd, t, 0, s>>>((float*)mom, (const double*)acc, rung, kick_state, n, rung_min,
-                                                        substep, log2_sub, dt, qq, qqf, nr, ctx->err_dev, pos,
+                                                        substep, log2_sub, kf, qq, qqf, nr, ctx->err_dev, pos,
                                                         drift_factor, L, slot);
     ++ctx->launches;
     if ((st = cuda_check(ctx, cudaGetLastError(), "rung kick-drift kernel")) != P3M_OK) return st;
@@ -510,16 +582,16 @@ static p3m_status rung_kick_impl(p3m_sr_ctx* ctx, void* mom, int mom_precision, 
   }
   if (mom_precision == 64 && acc_precision == 32)
     k_rung_kick<double, float><<<b, t, 0, s>>>((double*)mom, (const float*)acc, rung, kick_state, n, rung_min, substep,
-                                               log2_sub, dt, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
+                                               log2_sub, kf, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
   else if (mom_precision == 64 && acc_precision == 64)
     k_rung_kick<double, double><<<b, t, 0, s>>>((double*)mom, (const double*)acc, rung, kick_state, n, rung_min,
-                                                substep, log2_sub, dt, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
+                                                substep, log2_sub, kf, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
   else if (mom_precision == 32 && acc_precision == 32)
     k_rung_kick<float, float><<<b, t, 0, s>>>((float*)mom, (const float*)acc, rung, kick_state, n, rung_min, substep,
-                                              log2_sub, dt, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
+                                              log2_sub, kf, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
   else
     k_rung_kick<float, double><<<b, t, 0, s>>>((float*)mom, (const double*)acc, rung, kick_state, n, rung_min,
-                                               substep, log2_sub, dt, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
+                                               substep, log2_sub, kf, qq, rung_qqf(qq), nr, sy, ctx->err_dev);
   ++ctx->launches;
   if ((st = cuda_check(ctx, cudaGetLastError(), "rung kick kernel")) != P3M_OK) return st;
   report_latched(ctx);
