@@ -28,6 +28,7 @@ struct p3m_sr_ctx {
   int* scan_scratch = nullptr;
   int64_t scan_scratch_ints = 0;
   void* gather_tmp = nullptr;         // 32 n bytes
+  unsigned char* staged = nullptr;    // per radix tile: its particles are staged in gather_tmp
   int radix_passes = 0;
   int radix_bits[4] = {0, 0, 0, 0};
 

@@ -400,6 +400,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
     P3M_ALLOC(gt, 32 * n);
     ctx->gather_tmp = gt;
   }
+  P3M_ALLOC(ctx->staged, radix_blocks);
   P3M_ALLOC(ctx->active_flag, n);
   P3M_ALLOC(ctx->act_scan, n + 1);
   P3M_ALLOC(ctx->active_idx, n);
@@ -536,7 +537,7 @@ extern "C" void p3m_sr_destroy(p3m_sr_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream || true) cudaStreamSynchronize(ctx->stream);
   void* ptrs[] = {ctx->keys[0], ctx->keys[1], ctx->vals[0], ctx->vals[1], ctx->offsets, ctx->hist,
-                  ctx->scan_scratch, ctx->gather_tmp, ctx->active_flag, ctx->act_scan, ctx->active_idx,
+                  ctx->scan_scratch, ctx->gather_tmp, ctx->staged, ctx->active_flag, ctx->act_scan, ctx->active_idx,
                   ctx->tile_chunks, ctx->part_acc,
                   ctx->chunks, ctx->chunks_all, ctx->dev_small, ctx->pair_count,
                   ctx->rel4, ctx->org, ctx->abar4, ctx->abar_d, ctx->table, ctx->tab64, ctx->err_dev, ctx->drift_slots};
