@@ -714,6 +714,13 @@ __global__ void __launch_bounds__(kPThreads, VJP ? kSymVjpMinBlocks : kSymMinBlo
     const Chunk ch = chunk_at(a, ci);
     ChunkFrame F;
     load_chunk(a, rc, ch, lane, F);
+    {  // subtile planes along x that hold only smaller indices: the tile columns before the chunk's own
+      const int below = quot_small(F.g0[0], a.g.ns[0], a.g.inv_ns[0]) * a.g.ns[0] - F.g0[0] - F.elo[0];
+      if (below > 0 && F.g0[0] + F.elo[0] >= 0) {  // (those before column 0 wrap round to the last ones)
+        F.elo[0] += below;
+        F.ext[0] -= below;
+      }
+    }
     const float rx = F.valid ? F.pi.x : kSymPad, ry = F.valid ? F.pi.y : kSymPad, rz = F.valid ? F.pi.z : kSymPad;
     float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (VJP) {
