@@ -29,6 +29,7 @@ struct p3m_sr_ctx {
   int64_t scan_scratch_ints = 0;
   void* gather_tmp = nullptr;         // 32 n bytes
   unsigned char* staged = nullptr;    // per radix tile: its particles are staged in gather_tmp
+  int* unordered = nullptr;           // staged tiles of a sort (the word behind drift_slots; zero between sorts)
   int radix_passes = 0;
   int radix_bits[4] = {0, 0, 0, 0};
 

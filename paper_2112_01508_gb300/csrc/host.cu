@@ -415,7 +415,8 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->org, origin_count(ctx->geo));
   ctx->org_cap = origin_count(ctx->geo);
   P3M_ALLOC(ctx->err_dev, 1);
-  P3M_ALLOC(ctx->drift_slots, kMaxDrifts);
+  P3M_ALLOC(ctx->drift_slots, kMaxDrifts + 1);
+  ctx->unordered = (int*)(ctx->drift_slots + kMaxDrifts);
 #undef P3M_ALLOC
   if (cudaMallocHost((void**)&ctx->err_host, sizeof(int)) != cudaSuccess) {
     st = fail(ctx, P3M_ERR_OOM, "cudaMallocHost failed");
@@ -436,7 +437,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->scan_scratch, 0, sizeof(int) * ctx->scan_scratch_ints, ctx->stream),
                        "memset")) != P3M_OK)
     goto fail_alloc;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * kMaxDrifts, ctx->stream),
+  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * (kMaxDrifts + 1), ctx->stream),
                        "memset")) != P3M_OK)
     goto fail_alloc;
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small, 0, 16 * sizeof(int), ctx->stream), "memset")) != P3M_OK)
