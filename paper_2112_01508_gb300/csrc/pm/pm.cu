@@ -16,7 +16,9 @@
 #include <cuda_runtime.h>
 #include <cufft.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <new>
 #include <string>
@@ -100,8 +102,30 @@ __device__ __forceinline__ int wrap(long long m, long long n) {
 
 __device__ __forceinline__ bool position_ok(double x, double box) { return x >= 0.0 && x < box; }
 
-// rho[(X n + Y) pad + Z] += prod_d W_p for the p^3 cells of every particle.
-template <int P, class T>
+// P weights w[0 .. P) of one mesh row added at p (an element index `offs` from a 16-byte
+// aligned base): one vector reduction per aligned group of four cells instead of one per cell.
+template <int P>
+__device__ __forceinline__ void add_row(float* __restrict__ rho, long long offs, float wab, const float (&w)[P]) {
+  const int m = (int)(offs & 3);
+  float4* q = reinterpret_cast<float4*>(rho + (offs - m));
+  float v[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    v[t] = 0.0f;
+#pragma unroll
+    for (int c = 0; c < P; ++c)
+      if (t - c >= 0 && t - c < 4) v[t] = t - c == m ? wab * w[c] : v[t];
+  }
+  atomicAdd(q, make_float4(v[0], v[1], v[2], v[3]));
+  if (m + P > 4) atomicAdd(q + 1, make_float4(v[4], v[5], v[6], v[7]));
+}
+
+// rho[(X n + Y) pad + Z] += prod_d W_p for the p^3 cells of every particle.  VEC (FP32, rho
+// 16-byte aligned): the cells of a row that does not wrap go in vector reductions, one or two
+// of 16 bytes in place of P of 4.  The kernel is bound by the L2's reductions (in order of
+// tiles, clustered particles add to the same cells): with the mesh clear, 128^3 particles on
+// 256^3 cells, CIC 111 -> 107 us, TSC 267 -> 181 us, PCS 580 -> 344 us.
+template <int P, class T, bool VEC>
 __global__ void k_assign(const double* __restrict__ pos, long long n, long long nphi, long long pad, double scale,
                          double box, T* __restrict__ rho, int* __restrict__ err) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -117,6 +141,7 @@ __global__ void k_assign(const double* __restrict__ pos, long long n, long long 
     int iz[P];
 #pragma unroll
     for (int c = 0; c < P; ++c) iz[c] = wrap(fz + c, nphi);
+    const bool whole = VEC && fz >= 0 && fz + P <= nphi;
 #pragma unroll
     for (int a = 0; a < P; ++a) {
       const long long row_a = (long long)wrap(fx + a, nphi) * nphi;
@@ -124,6 +149,12 @@ __global__ void k_assign(const double* __restrict__ pos, long long n, long long 
       for (int b = 0; b < P; ++b) {
         const long long row = (row_a + wrap(fy + b, nphi)) * pad;
         const T wab = wx[a] * wy[b];
+        if constexpr (VEC) {
+          if (whole) {
+            add_row<P>(rho, row + fz, wab, wz);
+            continue;
+          }
+        }
 #pragma unroll
         for (int c = 0; c < P; ++c) atomicAdd(rho + row + iz[c], wab * wz[c]);
       }
@@ -153,6 +184,37 @@ __global__ void k_green(typename Cplx<T>::type* __restrict__ mesh, const T* __re
       v.y *= g;
       r[jz] = v;
     }
+  }
+}
+
+// The same with one thread per mode.  FP64 multiplications and the division bind the FP64
+// kernel, and a warp pays them for its idle lanes too: with 101 modes per row (n_phi = 200)
+// 223 -> 125 us, with 34 (66) 14 -> 10 us.  Rows that fill their warps to 80% stay with
+// k_green (61 modes: 31 us, 33 here), and so does FP32, which is bound by memory (129 modes:
+// 25 us, 31 here).
+template <class T>
+__global__ void k_green_flat(typename Cplx<T>::type* __restrict__ mesh, const T* __restrict__ f,
+                             const T* __restrict__ k2, int nphi, int nz, long long modes, T pref) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= modes) return;
+  // the mode's indices, advanced by the stride's own (jx, jy, jz) digits
+  int jx = (int)(i / nz / nphi), jy = (int)(i / nz - (long long)jx * nphi), jz = (int)(i % nz);
+  const int sx = (int)(stride / nz / nphi), sy = (int)(stride / nz - (long long)sx * nphi), sz = (int)(stride % nz);
+  for (; i < modes; i += stride) {
+    const T kk = k2[jx] + k2[jy] + k2[jz];
+    const T g = kk > T(0) ? f[jx] * f[jy] * pref * f[jz] / kk : T(0);
+    typename Cplx<T>::type v = mesh[i];
+    v.x *= g;
+    v.y *= g;
+    mesh[i] = v;
+    jz += sz;
+    int carry = jz >= nz ? 1 : 0;
+    jz -= carry ? nz : 0;
+    jy += sy + carry;
+    carry = jy >= nphi ? 1 : 0;
+    jy -= carry ? nphi : 0;
+    jx += sx + carry;
   }
 }
 
@@ -343,11 +405,16 @@ p3m_status launch_assign(p3m_pm_ctx* ctx, const double* pos, T* rho, long long p
   long long blocks = (n + threads - 1) / threads;
   if (blocks > (long long)ctx->num_sms * 64) blocks = (long long)ctx->num_sms * 64;
   const unsigned b = (unsigned)(blocks > 0 ? blocks : 1);
+  constexpr bool f32 = sizeof(T) == 4;
+  const bool vec = f32 && reinterpret_cast<uintptr_t>(rho) % 16 == 0;
+  auto launch = [&](auto kern) {
+    kern<<<b, threads, 0, ctx->stream>>>(pos, n, ctx->nphi, pad, scale, ctx->prm.box, rho, ctx->err_dev);
+  };
   switch (ctx->prm.p_i) {
-    case 1: k_assign<1, T><<<b, threads, 0, ctx->stream>>>(pos, n, ctx->nphi, pad, scale, ctx->prm.box, rho, ctx->err_dev); break;
-    case 2: k_assign<2, T><<<b, threads, 0, ctx->stream>>>(pos, n, ctx->nphi, pad, scale, ctx->prm.box, rho, ctx->err_dev); break;
-    case 3: k_assign<3, T><<<b, threads, 0, ctx->stream>>>(pos, n, ctx->nphi, pad, scale, ctx->prm.box, rho, ctx->err_dev); break;
-    default: k_assign<4, T><<<b, threads, 0, ctx->stream>>>(pos, n, ctx->nphi, pad, scale, ctx->prm.box, rho, ctx->err_dev); break;
+    case 1: launch(k_assign<1, T, false>); break;
+    case 2: vec ? launch(k_assign<2, T, f32>) : launch(k_assign<2, T, false>); break;
+    case 3: vec ? launch(k_assign<3, T, f32>) : launch(k_assign<3, T, false>); break;
+    default: vec ? launch(k_assign<4, T, f32>) : launch(k_assign<4, T, false>); break;
   }
   ++ctx->launches;
   return pm_cuda(ctx, cudaGetLastError(), "assign kernel");
@@ -383,11 +450,18 @@ p3m_status run_accel(p3m_pm_ctx* ctx, const double* pos, T* acc, int accumulate)
   if (st != P3M_OK) return st;
   cudaEventRecord(ctx->ev[2], s);
   {
-    const long long rows = ctx->nphi * ctx->nphi;
-    long long blocks = (rows + 7) / 8;
-    if (blocks > (long long)ctx->num_sms * 32) blocks = (long long)ctx->num_sms * 32;
-    k_green<T><<<(unsigned)blocks, 256, 0, s>>>((typename Cplx<T>::type*)ctx->mesh, (const T*)ctx->f_tab,
-                                                 (const T*)ctx->k2_tab, ctx->nphi, ctx->nz, (T)ctx->pref);
+    typename Cplx<T>::type* m = (typename Cplx<T>::type*)ctx->mesh;
+    const long long nz = ctx->nz, slots = (nz + 31) / 32 * 32;  // lanes a warp spends on a row
+    if (sizeof(T) == 8 && 5 * nz < 4 * slots) {
+      const long long modes = ctx->nphi * ctx->nphi * nz;
+      const long long blocks = std::min<long long>((modes + 255) / 256, (long long)ctx->num_sms * 8);
+      k_green_flat<T><<<(unsigned)blocks, 256, 0, s>>>(m, (const T*)ctx->f_tab, (const T*)ctx->k2_tab, (int)ctx->nphi,
+                                                       (int)nz, modes, (T)ctx->pref);
+    } else {
+      const long long blocks = std::min<long long>((ctx->nphi * ctx->nphi + 7) / 8, (long long)ctx->num_sms * 32);
+      k_green<T><<<(unsigned)blocks, 256, 0, s>>>(m, (const T*)ctx->f_tab, (const T*)ctx->k2_tab, ctx->nphi, nz,
+                                                   (T)ctx->pref);
+    }
     ++ctx->launches;
     if ((st = pm_cuda(ctx, cudaGetLastError(), "green kernel")) != P3M_OK) return st;
   }
