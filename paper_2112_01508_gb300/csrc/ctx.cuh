@@ -37,14 +37,13 @@ struct p3m_sr_ctx {
   int8_t* active_flag = nullptr;      // n
   int* act_scan = nullptr;            // n + 1
   int* active_idx = nullptr;          // n
-  int* tile_chunks = nullptr;         // n_tiles + 1 (chunks per row segment, scanned)
   float4* part_acc = nullptr;         // partial sums of split chunks (part_items work items x 32 lanes)
   int part_items = 0;
   p3m::Chunk* chunks = nullptr;       // receiver chunks of the last build_pairs
   p3m::Chunk* chunks_all = nullptr;   // chunks over all particles (vjp)
   int64_t max_chunks = 0;
-  int* dev_small = nullptr;           // [0] n_chunks, [1] n_chunks_all, [2] n_active,
-                                      // [3..7] work counters
+  int* dev_small = nullptr;           // [0] n_chunks, [1] n_chunks_all, [2] n_active, [3] and [4] work
+                                      // counters, [6..7] pair_count, [8..9] work words of k_build_chunks
   unsigned long long* pair_count = nullptr;
 
   // ---- per-call arrays ----

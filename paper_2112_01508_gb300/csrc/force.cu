@@ -211,34 +211,48 @@ __device__ __forceinline__ void segment_range(const int* __restrict__ offsets, c
   a1 = tile_start(offsets, act_scan, nsub3, t1);
 }
 
-__global__ void k_row_chunks(const int* __restrict__ offsets, const int* __restrict__ act_scan, int n_t, int nsub3,
-                             int* __restrict__ seg_chunks) {
-  const int64_t seg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The chunk list in one launch: each block takes 256 segments, scans their chunk counts and
+// reserves its part of the list with one atomic, so blocks follow one another in the order in
+// which they finish counting.  That is nearly the order of the segments (neighbouring chunks
+// share suppliers in L2), and nothing but that locality depends on it.  The last block to
+// finish publishes the count and clears the two work words, which are zero between launches.
+// (Counts, their scan in one or two launches and the list took 4 launches, 17 us at 128^3.)
+constexpr int kSegThreads = 256;
+__global__ void __launch_bounds__(kSegThreads) k_build_chunks(const int* __restrict__ offsets,
+                                                              const int* __restrict__ act_scan, int n_t, int nsub3,
+                                                              Chunk* __restrict__ chunks, int* work,
+                                                              int* __restrict__ n_chunks_out,
+                                                              int* __restrict__ n_active_out, int64_t n) {
+  __shared__ int warp_tot[kSegThreads / kWarp];
+  __shared__ int base;
+  const int64_t seg = (int64_t)blockIdx.x * kSegThreads + threadIdx.x;
   const int64_t nsegs = (int64_t)n_t * n_t * ((n_t + kChunkSpan - 1) / kChunkSpan);
-  if (seg > nsegs) return;
-  if (seg == nsegs) {
-    seg_chunks[nsegs] = 0;
-    return;
+  int a0 = 0, a1 = 0;
+  if (seg < nsegs) segment_range(offsets, act_scan, nsub3, n_t, seg, a0, a1);
+  const int c = (a1 - a0 + kChunk - 1) / kChunk;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int inc = c;
+  for (int o = 1; o < kWarp; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
   }
-  int a0, a1;
-  segment_range(offsets, act_scan, nsub3, n_t, seg, a0, a1);
-  seg_chunks[seg] = (a1 - a0 + kChunk - 1) / kChunk;
-}
-
-__global__ void k_write_chunks(const int* __restrict__ offsets, const int* __restrict__ act_scan, int n_t, int nsub3,
-                               const int* __restrict__ seg_chunks, Chunk* __restrict__ chunks,
-                               int* __restrict__ n_chunks_out, int* __restrict__ n_active_out, int64_t n) {
-  const int64_t seg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nsegs = (int64_t)n_t * n_t * ((n_t + kChunkSpan - 1) / kChunkSpan);
-  if (seg == 0) {
-    *n_chunks_out = seg_chunks[nsegs];
-    if (n_active_out) *n_active_out = act_scan ? act_scan[n] : (int)n;
+  if (lane == kWarp - 1) warp_tot[warp] = inc;
+  __syncthreads();
+  int at = inc - c;
+  for (int w = 0; w < warp; ++w) at += warp_tot[w];
+  if (threadIdx.x == kSegThreads - 1) {
+    base = atomicAdd(&work[0], at + c);
+    __threadfence();
+    if (atomicAdd(&work[1], 1) == (int)gridDim.x - 1) {
+      __threadfence();
+      *n_chunks_out = atomicExch(&work[0], 0);
+      work[1] = 0;
+      if (n_active_out) *n_active_out = act_scan ? act_scan[n] : (int)n;
+    }
   }
-  if (seg >= nsegs) return;
-  int a0, a1;
-  segment_range(offsets, act_scan, nsub3, n_t, seg, a0, a1);
-  Chunk* out = chunks + seg_chunks[seg];
-  for (int k = 0; a0 + k * kChunk < a1; ++k) {
+  __syncthreads();
+  Chunk* out = chunks + base + at;
+  for (int k = 0; k < c; ++k) {
     const int s0 = a0 + k * kChunk;
     out[k] = Chunk{s0, min(kChunk, a1 - s0)};
   }
@@ -1253,19 +1267,10 @@ static p3m_status build_chunks(p3m_sr_ctx* ctx, const int* act_scan, Chunk* chun
   cudaStream_t s = ctx->stream;
   const int n_t = ctx->geo.n_t;
   const int64_t rows = (int64_t)n_t * n_t * ((n_t + kChunkSpan - 1) / kChunkSpan);  // segments
-  k_row_chunks<<<blocks_for(rows + 1, 128), 128, 0, s>>>(ctx->offsets, act_scan, n_t, ctx->geo.nsub3,
-                                                         ctx->tile_chunks);
+  k_build_chunks<<<blocks_for(rows, kSegThreads), kSegThreads, 0, s>>>(
+      ctx->offsets, act_scan, n_t, ctx->geo.nsub3, chunks, ctx->dev_small + 8, n_chunks_dev, n_active_dev, ctx->n);
   ++ctx->launches;
-  p3m_status st = cuda_check(ctx, cudaGetLastError(), "row chunk kernel");
-  if (st != P3M_OK) return st;
-  st = cuda_check(ctx, scan_exclusive_i32(ctx->tile_chunks, ctx->tile_chunks, rows + 1, ctx->scan_scratch,
-                                          ctx->scan_scratch_ints, s, &ctx->launches), "chunk scan");
-  if (st != P3M_OK) return st;
-  k_write_chunks<<<blocks_for(rows, 128), 128, 0, s>>>(ctx->offsets, act_scan, n_t, ctx->geo.nsub3,
-                                                        ctx->tile_chunks, chunks, n_chunks_dev, n_active_dev,
-                                                        ctx->n);
-  ++ctx->launches;
-  return cuda_check(ctx, cudaGetLastError(), "write chunks kernel");
+  return cuda_check(ctx, cudaGetLastError(), "chunk kernel");
 }
 
 p3m_status ensure_all_chunks(p3m_sr_ctx* ctx) {
@@ -1290,6 +1295,11 @@ static TraversalArgs base_args(p3m_sr_ctx* ctx) {
   a.n_drift = ctx->n_drift;
   a.err = ctx->err_dev;
   return a;
+}
+
+// The work counters of the traversals and the pair count, in one memset.
+static p3m_status clear_counters(p3m_sr_ctx* ctx) {
+  return cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 3, 0, 5 * sizeof(int), ctx->stream), "memset");
 }
 
 static p3m_status prepare_rel4(p3m_sr_ctx* ctx, const double* pos) {
@@ -1347,11 +1357,9 @@ extern "C" p3m_status p3m_sr_forces(p3m_sr_ctx* ctx, const double* pos, int prec
   p3m_status st = poll_latched(ctx);
   if (st != P3M_OK) return st;
   cudaStream_t s = ctx->stream;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->pair_count, 0, sizeof(unsigned long long), s), "memset")) != P3M_OK)
-    return st;
+  if ((st = clear_counters(ctx)) != P3M_OK) return st;
   if (ctx->n == 0) return P3M_OK;
   if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 3, 0, sizeof(int), s), "memset")) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
   a.chunks = ctx->chunks;
@@ -1425,11 +1433,9 @@ extern "C" p3m_status p3m_sr_forces_tabulated(p3m_sr_ctx* ctx, const double* pos
       return st;
     ctx->table_bits = table_bits;
   }
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->pair_count, 0, sizeof(unsigned long long), s), "memset")) != P3M_OK)
-    return st;
+  if ((st = clear_counters(ctx)) != P3M_OK) return st;
   if (ctx->n == 0) return P3M_OK;
   if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 3, 0, sizeof(int), s), "memset")) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
   a.chunks = ctx->chunks;
@@ -1479,8 +1485,7 @@ extern "C" p3m_status p3m_sr_vjp(p3m_sr_ctx* ctx, const double* pos, int precisi
   if (st != P3M_OK) return st;
   cudaStream_t s = ctx->stream;
   const int64_t n = ctx->n;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->pair_count, 0, sizeof(unsigned long long), s), "memset")) != P3M_OK)
-    return st;
+  if ((st = clear_counters(ctx)) != P3M_OK) return st;
   if (n == 0) return P3M_OK;
   if (precision == 32 && !ctx->abar4) {
     if ((st = cuda_check(ctx, cudaMalloc((void**)&ctx->abar4, sizeof(float4) * ctx->cap), "cudaMalloc(abar4)")) != P3M_OK)
@@ -1500,7 +1505,6 @@ extern "C" p3m_status p3m_sr_vjp(p3m_sr_ctx* ctx, const double* pos, int precisi
                                                    ctx->abar_d);
   ++ctx->launches;
   if ((st = cuda_check(ctx, cudaGetLastError(), "abar kernel")) != P3M_OK) return st;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 4, 0, sizeof(int), s), "memset")) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
   a.chunks = ctx->chunks_all;
@@ -1555,8 +1559,7 @@ struct NoallocLayout {
   static constexpr int64_t bad = wpos + noalloc_align(8 * 3 * kNoallocMaxN);
   static constexpr int64_t pos = bad + noalloc_align(kNoallocMaxN);
   static constexpr int64_t rel4 = pos + noalloc_align(8 * 3 * kNoallocMaxN);
-  static constexpr int64_t rows = rel4 + noalloc_align(16 * kNoallocMaxN);
-  static constexpr int64_t chunks = rows + noalloc_align(4 * (kNoallocMaxRows + 1));
+  static constexpr int64_t chunks = rel4 + noalloc_align(16 * kNoallocMaxN);
   static constexpr int64_t acc = chunks + noalloc_align(8 * kNoallocMaxChunks);
   static constexpr int64_t small = acc + noalloc_align(4 * 3 * kNoallocMaxN);
   static constexpr int64_t total = small + noalloc_align(64);
@@ -1677,7 +1680,6 @@ extern "C" p3m_status p3m_sr_forces_noalloc(const p3m_sr_params* params, void* c
   unsigned char* bad = base + Lay::bad;
   double* spos = (double*)(base + Lay::pos);
   float4* rel4 = (float4*)(base + Lay::rel4);
-  int* rows = (int*)(base + Lay::rows);
   Chunk* chunks = (Chunk*)(base + Lay::chunks);
   float* acc = (float*)(base + Lay::acc);
   int* small = (int*)(base + Lay::small);  // [0] n_chunks, [1] counter, [2] k_bin's error word (unused: the
@@ -1720,11 +1722,8 @@ extern "C" p3m_status p3m_sr_forces_noalloc(const p3m_sr_params* params, void* c
   if (!ok(cudaGetLastError())) return P3M_ERR_CUDA;
   // receiver chunks (all particles active)
   const int64_t nrows = (int64_t)g.n_t * g.n_t * ((g.n_t + kChunkSpan - 1) / kChunkSpan);  // segments
-  k_row_chunks<<<(unsigned)((nrows + 1 + 127) / 128), 128, 0, s>>>(offsets, nullptr, g.n_t, g.nsub3, rows);
-  if (!ok(cudaGetLastError())) return P3M_ERR_CUDA;
-  if (!ok(scan_exclusive_i32(rows, rows, nrows + 1, scan, kNoallocScanInts, s, &launches))) return P3M_ERR_CUDA;
-  k_write_chunks<<<(unsigned)((nrows + 127) / 128), 128, 0, s>>>(offsets, nullptr, g.n_t, g.nsub3, rows, chunks,
-                                                                 small + 0, nullptr, n);
+  k_build_chunks<<<(unsigned)((nrows + kSegThreads - 1) / kSegThreads), kSegThreads, 0, s>>>(
+      offsets, nullptr, g.n_t, g.nsub3, chunks, small + 8, small + 0, nullptr, n);
   if (!ok(cudaGetLastError())) return P3M_ERR_CUDA;
   // pair forces in the sorted order, then back to the caller's order
   static SeriesConsts series = make_series();

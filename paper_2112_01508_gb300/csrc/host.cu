@@ -404,13 +404,12 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->active_flag, n);
   P3M_ALLOC(ctx->act_scan, n + 1);
   P3M_ALLOC(ctx->active_idx, n);
-  P3M_ALLOC(ctx->tile_chunks, ctx->n_tiles + 1);
   ctx->part_items = (int)std::min<int64_t>(kPartItems, ctx->max_chunks * kPartItemsPerChunk);
   P3M_ALLOC(ctx->part_acc, (int64_t)ctx->part_items * kChunk);
   P3M_ALLOC(ctx->chunks, ctx->max_chunks);
   P3M_ALLOC(ctx->chunks_all, ctx->max_chunks);
   P3M_ALLOC(ctx->dev_small, 16);
-  P3M_ALLOC(ctx->pair_count, 2);
+  ctx->pair_count = (unsigned long long*)(ctx->dev_small + 6);
   P3M_ALLOC(ctx->rel4, n);
   P3M_ALLOC(ctx->org, origin_count(ctx->geo));
   ctx->org_cap = origin_count(ctx->geo);
@@ -441,9 +440,6 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
                        "memset")) != P3M_OK)
     goto fail_alloc;
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small, 0, 16 * sizeof(int), ctx->stream), "memset")) != P3M_OK)
-    goto fail_alloc;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->pair_count, 0, 2 * sizeof(unsigned long long), ctx->stream),
-                       "memset")) != P3M_OK)
     goto fail_alloc;
   if ((st = fill_origins(ctx)) != P3M_OK) goto fail_alloc;
   *out = ctx;
@@ -539,8 +535,7 @@ extern "C" void p3m_sr_destroy(p3m_sr_ctx* ctx) {
   if (ctx->stream || true) cudaStreamSynchronize(ctx->stream);
   void* ptrs[] = {ctx->keys[0], ctx->keys[1], ctx->vals[0], ctx->vals[1], ctx->offsets, ctx->hist,
                   ctx->scan_scratch, ctx->gather_tmp, ctx->staged, ctx->active_flag, ctx->act_scan, ctx->active_idx,
-                  ctx->tile_chunks, ctx->part_acc,
-                  ctx->chunks, ctx->chunks_all, ctx->dev_small, ctx->pair_count,
+                  ctx->part_acc, ctx->chunks, ctx->chunks_all, ctx->dev_small,
                   ctx->rel4, ctx->org, ctx->abar4, ctx->abar_d, ctx->table, ctx->tab64, ctx->err_dev, ctx->drift_slots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
