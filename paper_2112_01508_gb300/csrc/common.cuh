@@ -176,22 +176,24 @@ __global__ void k_fill_origins(Geometry g, double* __restrict__ org);
 
 // ---- kernels of sort.cu launched from other translation units ---------------
 constexpr int kRadixThreadsPublic = 256;
-#ifndef P3M_RADIX_STEPS
-#define P3M_RADIX_STEPS 8  // radix items per lane (8: 2048-item tiles, 7% faster than 4096 at 128^3, 26% at 512^3)
-#endif
-constexpr int kRadixTilePublic = kRadixThreadsPublic * P3M_RADIX_STEPS;  // items per radix block
+constexpr int kRadixStepsPublic = 8;  // items per lane (2048-item tiles: 7% faster than 4096 at 128^3, 26% at 512^3)
+constexpr int kRadixTilePublic = kRadixThreadsPublic * kRadixStepsPublic;
+constexpr int kRadixSmallSteps = 2;   // ... of sets of at most kRadixSmallN particles
+constexpr int64_t kRadixSmallN = 152 * kRadixTilePublic;  // a long tile per SM
+constexpr int kRadixSmallTile = kRadixThreadsPublic * kRadixSmallSteps;
+constexpr int kOffsetsLead = 4;       // words in front of the subtile offsets (cleared with them)
 __global__ void k_bin(const double* __restrict__ pos, int64_t n, Geometry g, int* __restrict__ keys,
                       int* __restrict__ vals, int* __restrict__ counts, int* __restrict__ err);
 __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift, int bits, int* __restrict__ hist,
                              int nblocks);
-__global__ void k_radix_scatter(const int* __restrict__ keys_in, const int* __restrict__ vals_in,
-                                int* __restrict__ keys_out, int* __restrict__ vals_out, int64_t n, int shift,
-                                int bits, const int* __restrict__ hist, int nblocks, int* __restrict__ hist_next,
-                                int shift_next, int bits_next);
 __global__ void k_gather_pos(const double* __restrict__ src, const int* __restrict__ perm, int64_t n,
                              double* __restrict__ dst);
 
 // ---- launch helpers (host) --------------------------------------------------
+
+// One pass of the stable radix sort over tiles of kRadixTilePublic, histogram scanned before.
+void launch_radix_scatter(int nblocks, cudaStream_t s, const int* keys_in, const int* vals_in, int* keys_out, int* vals_out,
+                          int64_t n, int shift, int bits, const int* hist);
 
 // Exclusive scan of n int32 values (in may equal out).  Returns cudaError.
 // scratch: scratch_ints >= scan_scratch_ints(n) ints whose last int is zero before
@@ -199,6 +201,10 @@ __global__ void k_gather_pos(const double* __restrict__ src, const int* __restri
 // *launches.
 cudaError_t scan_exclusive_i32(const int* in, int* out, int64_t n, int* scratch, int64_t scratch_ints, cudaStream_t s,
                                int64_t* launches);
+// Two exclusive scans in place in the launches of one (v2 may be empty).  scratch_ints as for
+// the longer one, twice.
+cudaError_t scan_exclusive_i32_pair(int* v1, int64_t n1, int* v2, int64_t n2, int* scratch, int64_t scratch_ints,
+                                    cudaStream_t s, int64_t* launches);
 // Scratch (ints) needed by scan_exclusive_i32 for n elements.
 int64_t scan_scratch_ints(int64_t n);
 

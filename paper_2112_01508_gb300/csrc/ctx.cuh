@@ -19,7 +19,7 @@ struct p3m_sr_ctx {
   // ---- sort scratch ----
   int* keys[2] = {nullptr, nullptr};  // radix double buffers
   int* vals[2] = {nullptr, nullptr};
-  int* offsets = nullptr;             // S + 1 (histogram, scanned in place)
+  int* offsets = nullptr;             // S + 1 (histogram, scanned in place), behind kOffsetsLead words
   int64_t offsets_cap = 0;            // allocated ints of offsets
   int* cell = nullptr;                // sorted subtile ids (aliases keys[k])
   int* perm = nullptr;                // sorted -> input index (aliases vals[k])
@@ -28,8 +28,7 @@ struct p3m_sr_ctx {
   int* scan_scratch = nullptr;
   int64_t scan_scratch_ints = 0;
   void* gather_tmp = nullptr;         // 32 n bytes
-  unsigned char* staged = nullptr;    // per radix tile: its particles are staged in gather_tmp
-  int* unordered = nullptr;           // staged tiles of a sort (the word behind drift_slots; zero between sorts)
+  unsigned char* staged = nullptr;    // per kRadixSmallTile particles: they are staged in gather_tmp
   int radix_passes = 0;
   int radix_bits[4] = {0, 0, 0, 0};
 

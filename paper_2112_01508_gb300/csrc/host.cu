@@ -77,10 +77,10 @@ __global__ void k_scan_reduce(const int* __restrict__ in, int64_t n, int* __rest
   }
 }
 
-__global__ void k_scan_tile(const int* in, int* out, int64_t n, const int* __restrict__ offs) {
+__device__ __forceinline__ void scan_tile(const int* in, int* out, int64_t n, int block, const int* offs) {
   __shared__ int tile[kScanTile + kScanTile / 32];
   __shared__ int warp_tot[kScanThreads / kWarp];
-  int64_t base = (int64_t)blockIdx.x * kScanTile;
+  int64_t base = (int64_t)block * kScanTile;
   for (int k = 0; k < kScanItems; ++k) {
     int li = k * kScanThreads + threadIdx.x;
     int64_t i = base + li;
@@ -105,7 +105,7 @@ __global__ void k_scan_tile(const int* in, int* out, int64_t n, const int* __res
   __syncthreads();
   int wpre = 0;
   for (int w = 0; w < warp; ++w) wpre += warp_tot[w];
-  int run = wpre + inc - tot + (offs ? offs[blockIdx.x] : 0);
+  int run = wpre + inc - tot + (offs ? offs[block] : 0);
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     tile[smem_pad(threadIdx.x * kScanItems + k)] = run;
@@ -117,6 +117,10 @@ __global__ void k_scan_tile(const int* in, int* out, int64_t n, const int* __res
     int64_t i = base + li;
     if (i < n) out[i] = tile[smem_pad(li)];
   }
+}
+
+__global__ void k_scan_tile(const int* in, int* out, int64_t n, const int* __restrict__ offs) {
+  scan_tile(in, out, n, blockIdx.x, offs);
 }
 
 // Exclusive scan of the nb <= kScanTile values of v in place, by one block.
@@ -178,6 +182,53 @@ __global__ void k_scan_reduce_last(const int* __restrict__ in, int64_t n, int* s
   }
 }
 
+// Two arrays at once: blocks [0, a.nb) take the tiles of a, the rest those of b.
+struct ScanPart {
+  int* v;
+  int64_t n;
+  int nb;
+  int* sums;  // tile sums (scanned by the block that finishes last)
+};
+
+__global__ void k_scan_reduce_last2(ScanPart a, ScanPart b, int* ticket) {
+  __shared__ int warp_sums[kScanThreads / kWarp];
+  __shared__ bool last;
+  const bool first = (int)blockIdx.x < a.nb;
+  const int tile = first ? blockIdx.x : blockIdx.x - a.nb;
+  const int* v = first ? a.v : b.v;
+  const int64_t n = first ? a.n : b.n;
+  const int64_t base = (int64_t)tile * kScanTile;
+  int s = 0;
+  for (int k = 0; k < kScanItems; ++k) {
+    const int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
+    if (i < n) s += v[i];
+  }
+  s = __reduce_add_sync(0xffffffffu, s);
+  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int t = 0;
+    for (int w = 0; w < kScanThreads / kWarp; ++w) t += warp_sums[w];
+    (first ? a.sums : b.sums)[tile] = t;
+    __threadfence();
+    last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    block_scan_small(a.sums, a.nb);
+    __syncthreads();
+    block_scan_small(b.sums, b.nb);
+    if (threadIdx.x == 0) *ticket = 0;
+  }
+}
+
+__global__ void k_scan_tile2(ScanPart a, ScanPart b) {
+  const bool first = (int)blockIdx.x < a.nb;
+  const int tile = first ? blockIdx.x : blockIdx.x - a.nb;
+  scan_tile(first ? a.v : b.v, first ? a.v : b.v, first ? a.n : b.n, tile, first ? a.sums : b.sums);
+}
+
 int64_t scan_scratch_ints(int64_t n) {
   int64_t total = 0;
   int64_t m = n;
@@ -209,6 +260,25 @@ static cudaError_t scan_rec(const int* in, int* out, int64_t n, int* scratch, in
     if (e != cudaSuccess) return e;
   }
   k_scan_tile<<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, sums);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t scan_exclusive_i32_pair(int* v1, int64_t n1, int* v2, int64_t n2, int* scratch, int64_t scratch_ints,
+                                    cudaStream_t s, int64_t* launches) {
+  const int64_t nb1 = (n1 + kScanTile - 1) / kScanTile, nb2 = (n2 + kScanTile - 1) / kScanTile;
+  if (nb1 > kScanTile || nb2 > kScanTile || nb1 == 0 || nb2 == 0) {
+    cudaError_t e = scan_exclusive_i32(v1, v1, n1, scratch, scratch_ints, s, launches);
+    return e != cudaSuccess ? e : scan_exclusive_i32(v2, v2, n2, scratch, scratch_ints, s, launches);
+  }
+  const unsigned blocks = (unsigned)(nb1 + nb2);
+  const bool single = nb1 == 1 && nb2 == 1;  // no tile sums
+  const ScanPart a{v1, n1, (int)nb1, single ? nullptr : scratch}, b{v2, n2, (int)nb2, single ? nullptr : scratch + nb1};
+  if (!single) {
+    k_scan_reduce_last2<<<blocks, kScanThreads, 0, s>>>(a, b, scratch + scratch_ints - 1);
+    ++*launches;
+  }
+  k_scan_tile2<<<blocks, kScanThreads, 0, s>>>(a, b);
   ++*launches;
   return cudaGetLastError();
 }
@@ -378,9 +448,10 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   const int64_t n = ctx->n;
   const int64_t S = ctx->geo.S;
   setup_radix(ctx);
-  int64_t radix_blocks = (n + kRadixTilePublic - 1) / kRadixTilePublic;
+  const int64_t radix_blocks = std::max<int64_t>((n + kRadixTilePublic - 1) / kRadixTilePublic,
+                                                 (std::min<int64_t>(n, kRadixSmallN) + kRadixSmallTile - 1) / kRadixSmallTile);
   ctx->hist_ints = 1024 * (radix_blocks > 0 ? radix_blocks : 1);
-  ctx->scan_scratch_ints = scan_scratch_ints(scan_length(ctx));
+  ctx->scan_scratch_ints = 2 * scan_scratch_ints(scan_length(ctx));
   ctx->offsets_cap = S + 1;
   ctx->max_chunks = std::min<int64_t>(n, ctx->n_tiles) + (n + kChunk - 1) / kChunk + 1;
 
@@ -392,7 +463,11 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->keys[1], n);
   P3M_ALLOC(ctx->vals[0], n);
   P3M_ALLOC(ctx->vals[1], n);
-  P3M_ALLOC(ctx->offsets, S + 1);
+  {
+    int* o = nullptr;
+    P3M_ALLOC(o, S + 1 + kOffsetsLead);
+    ctx->offsets = o + kOffsetsLead;
+  }
   P3M_ALLOC(ctx->hist, 2 * ctx->hist_ints);  // this radix pass's digit counts and the next pass's
   P3M_ALLOC(ctx->scan_scratch, ctx->scan_scratch_ints);
   {
@@ -400,7 +475,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
     P3M_ALLOC(gt, 32 * n);
     ctx->gather_tmp = gt;
   }
-  P3M_ALLOC(ctx->staged, radix_blocks);
+  P3M_ALLOC(ctx->staged, (n + kRadixTilePublic - 1) / kRadixTilePublic * (kRadixTilePublic / kRadixSmallTile));
   P3M_ALLOC(ctx->active_flag, n);
   P3M_ALLOC(ctx->act_scan, n + 1);
   P3M_ALLOC(ctx->active_idx, n);
@@ -414,8 +489,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   P3M_ALLOC(ctx->org, origin_count(ctx->geo));
   ctx->org_cap = origin_count(ctx->geo);
   P3M_ALLOC(ctx->err_dev, 1);
-  P3M_ALLOC(ctx->drift_slots, kMaxDrifts + 1);
-  ctx->unordered = (int*)(ctx->drift_slots + kMaxDrifts);
+  P3M_ALLOC(ctx->drift_slots, kMaxDrifts);
 #undef P3M_ALLOC
   if (cudaMallocHost((void**)&ctx->err_host, sizeof(int)) != cudaSuccess) {
     st = fail(ctx, P3M_ERR_OOM, "cudaMallocHost failed");
@@ -436,7 +510,7 @@ extern "C" p3m_status p3m_sr_create(const p3m_sr_params* params, void* cuda_stre
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->scan_scratch, 0, sizeof(int) * ctx->scan_scratch_ints, ctx->stream),
                        "memset")) != P3M_OK)
     goto fail_alloc;
-  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * (kMaxDrifts + 1), ctx->stream),
+  if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * kMaxDrifts, ctx->stream),
                        "memset")) != P3M_OK)
     goto fail_alloc;
   if ((st = cuda_check(ctx, cudaMemsetAsync(ctx->dev_small, 0, 16 * sizeof(int), ctx->stream), "memset")) != P3M_OK)
@@ -485,12 +559,12 @@ extern "C" p3m_status p3m_sr_set_subtiles(p3m_sr_ctx* ctx, const int* n_sub) {
   ctx->prm = p;
   setup_geometry(ctx);
   // per-subtile offsets and the scan scratch grow with S; cudaFree waits for queued work
-  int64_t scan_ints = scan_scratch_ints(scan_length(ctx));
+  int64_t scan_ints = 2 * scan_scratch_ints(scan_length(ctx));
   int* new_offsets = nullptr;
   int* new_scan = nullptr;
   double* new_org = nullptr;
   const int64_t n_org = origin_count(ctx->geo);
-  if (S + 1 > ctx->offsets_cap && (st = alloc(ctx, &new_offsets, S + 1, "offsets")) != P3M_OK) goto restore;
+  if (S + 1 > ctx->offsets_cap && (st = alloc(ctx, &new_offsets, S + 1 + kOffsetsLead, "offsets")) != P3M_OK) goto restore;
   if (scan_ints > ctx->scan_scratch_ints && (st = alloc(ctx, &new_scan, scan_ints, "scan_scratch")) != P3M_OK) {
     cudaFree(new_offsets);
     goto restore;
@@ -506,8 +580,8 @@ extern "C" p3m_status p3m_sr_set_subtiles(p3m_sr_ctx* ctx, const int* n_sub) {
     ctx->org_cap = n_org;
   }
   if (new_offsets) {
-    cudaFree(ctx->offsets);
-    ctx->offsets = new_offsets;
+    cudaFree(ctx->offsets - kOffsetsLead);
+    ctx->offsets = new_offsets + kOffsetsLead;
     ctx->offsets_cap = S + 1;
   }
   if (new_scan) {
@@ -533,7 +607,8 @@ restore:
 extern "C" void p3m_sr_destroy(p3m_sr_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream || true) cudaStreamSynchronize(ctx->stream);
-  void* ptrs[] = {ctx->keys[0], ctx->keys[1], ctx->vals[0], ctx->vals[1], ctx->offsets, ctx->hist,
+  void* ptrs[] = {ctx->keys[0], ctx->keys[1], ctx->vals[0], ctx->vals[1],
+                  ctx->offsets ? ctx->offsets - kOffsetsLead : nullptr, ctx->hist,
                   ctx->scan_scratch, ctx->gather_tmp, ctx->staged, ctx->active_flag, ctx->act_scan, ctx->active_idx,
                   ctx->part_acc, ctx->chunks, ctx->chunks_all, ctx->dev_small,
                   ctx->rel4, ctx->org, ctx->abar4, ctx->abar_d, ctx->table, ctx->tab64, ctx->err_dev, ctx->drift_slots};

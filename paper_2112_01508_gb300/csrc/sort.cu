@@ -17,9 +17,13 @@ namespace p3m {
 
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / kWarp;
-constexpr int kRadixSteps = P3M_RADIX_STEPS;              // items per lane
-constexpr int kRadixTile = kRadixThreads * kRadixSteps;   // items per block
-static_assert(kRadixThreads == kRadixThreadsPublic && kRadixTile == kRadixTilePublic, "radix tiling");
+static_assert(kRadixThreads == kRadixThreadsPublic, "radix tiling");
+// Items per lane of a radix block: a serial chain of rounds, which is what a small set waits
+// for, so up to kRadixSmallN particles (one long tile per SM) the tiles are a quarter as
+// long.  A whole nearly sorted sort with long -> short tiles: 32,768 particles 62 -> 55 us,
+// 131,072 73 -> 62, 311,296 71 -> 66, 524,288 75 -> 78, 1,048,576 99 -> 112.
+template <int STEPS>
+constexpr int kTileOf = kRadixThreads * STEPS;
 
 // Subtile id of particle i: g_d = min(floor(x_d M_d / L), M_d - 1) with one correctly
 // rounded multiply; a coordinate outside [0, L) (or NaN) is binned as 0 and sets *bad.
@@ -87,6 +91,7 @@ struct StageArgs {
   int always;               // stage every tile (in-place sorts)
   int* unordered;           // number of staged tiles (zero before the sort)
   int nblocks;              // radix tiles
+  float* drift_slots;       // cleared by the binning kernel
   int phased;               // the other one-word arrays of an unordered input go to k_gather_phases
 };
 
@@ -99,21 +104,26 @@ __device__ __forceinline__ void stage_record(const StageArgs& st, int64_t i, con
   st.rec[2 * i + 1] = make_double2(x[2], __longlong_as_double((long long)w));
 }
 
-// k_bin over radix tiles of kRadixTile particles, which also counts the digits of
+// k_bin over radix tiles of kTileOf<STEPS> particles, which also counts the digits of
 // the first radix pass (bits low bits of the id) per tile: hist[d nblocks + tile].
+template <int STEPS>
 __global__ void __launch_bounds__(256) k_bin_tile(const double* __restrict__ pos, int64_t n, Geometry g,
                                                   int* __restrict__ keys, int* __restrict__ vals,
                                                   int* __restrict__ counts, int* __restrict__ err,
                                                   int* __restrict__ hist, int bits, int nblocks,
+                                                  int* __restrict__ hist_next, int next_ints,
                                                   const __grid_constant__ StageArgs st) {
   __shared__ int cnt[1024];
+  for (int d = threadIdx.x; d < next_ints; d += blockDim.x)  // the next pass's counts, cleared
+    hist_next[(int64_t)blockIdx.x * next_ints + d] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < kMaxDrifts) st.drift_slots[threadIdx.x] = 0.0f;  // no displacement since this sort
   const int radix = 1 << bits, mask = radix - 1;
   for (int d = threadIdx.x; d < radix; d += blockDim.x) cnt[d] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int64_t base = (int64_t)blockIdx.x * kRadixTile;
+  const int64_t base = (int64_t)blockIdx.x * kTileOf<STEPS>;
   bool any_bad = false, staged = false;
-  for (int k = 0; k < kRadixSteps; ++k) {
+  for (int k = 0; k < STEPS; ++k) {
     const int64_t i = base + (int64_t)k * kRadixThreads + threadIdx.x;
     const bool valid = i < n;
     int id = 0;
@@ -130,10 +140,9 @@ __global__ void __launch_bounds__(256) k_bin_tile(const double* __restrict__ pos
       const int next = __shfl_down_sync(0xffffffffu, id, 1);
       const bool far = valid && lane < 31 && abs(next - id) > kStageTiles * g.nsub3;
       staged = st.rec && (__syncthreads_count(far) > kRadixThreads / 4 || st.always);
-      if (threadIdx.x == 0) {
-        st.staged[blockIdx.x] = staged ? 1 : 0;
-        if (staged && st.phased) atomicAdd(st.unordered, 1);
-      }
+      constexpr int kFlags = STEPS / kRadixSmallSteps;  // one per kRadixSmallSteps rounds
+      if (threadIdx.x < kFlags) st.staged[blockIdx.x * kFlags + threadIdx.x] = staged ? 1 : 0;
+      if (threadIdx.x == 0 && staged && st.phased) atomicAdd(st.unordered, 1);
     }
     if (staged && valid) stage_record(st, i, x);
     const unsigned peers = __match_any_sync(0xffffffffu, valid ? id : -1 - lane);
@@ -152,9 +161,9 @@ __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift,
   const int radix = 1 << bits;
   for (int d = threadIdx.x; d < radix; d += blockDim.x) cnt[d] = 0;
   __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * kRadixTile;
+  int64_t base = (int64_t)blockIdx.x * kRadixTilePublic;
   const int mask = radix - 1;
-  for (int k = 0; k < kRadixSteps; ++k) {
+  for (int k = 0; k < kRadixTilePublic / kRadixThreads; ++k) {
     int64_t i = base + (int64_t)k * kRadixThreads + threadIdx.x;
     if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & mask], 1);
   }
@@ -170,6 +179,7 @@ __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift,
 // hist_next (nullable, zeroed before the launch): the digit counts of the next pass
 // (bits_next bits from shift_next) per output tile, accumulated here with one atomic
 // per distinct (digit, tile) of each warp, so that pass needs no histogram kernel.
+template <int STEPS>
 __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     const int* __restrict__ keys_in, const int* __restrict__ vals_in, int* __restrict__ keys_out,
     int* __restrict__ vals_out, int64_t n, int shift, int bits, const int* __restrict__ hist, int nblocks,
@@ -177,18 +187,18 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
   __shared__ int wcnt[kRadixWarps][kMaxRadix];  // per-warp digit counts; later the staged tile
   __shared__ int bstart[kMaxRadix];             // first position of each digit in the block's tile
   __shared__ int wtot[kRadixWarps];
-  static_assert(kRadixWarps * kMaxRadix >= 2 * kRadixTile, "staging area");
+  static_assert(kRadixWarps * kMaxRadix >= 2 * kTileOf<STEPS>, "staging area");
   const int radix = 1 << bits;
   const int mask = radix - 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int d = lane; d < radix; d += 32) wcnt[warp][d] = 0;
   __syncwarp();
-  const int64_t tile0 = (int64_t)blockIdx.x * kRadixTile;
-  const int64_t wbase = tile0 + (int64_t)warp * (kRadixSteps * kWarp);
+  const int64_t tile0 = (int64_t)blockIdx.x * kTileOf<STEPS>;
+  const int64_t wbase = tile0 + (int64_t)warp * (STEPS * kWarp);
   const unsigned lt = (1u << lane) - 1u;
-  int key[kRadixSteps], val[kRadixSteps], rank[kRadixSteps];
+  int key[STEPS], val[STEPS], rank[STEPS];
 #pragma unroll
-  for (int k = 0; k < kRadixSteps; ++k) {
+  for (int k = 0; k < STEPS; ++k) {
     int64_t i = wbase + k * kWarp + lane;
     bool valid = i < n;
     key[k] = valid ? keys_in[i] : 0;
@@ -242,19 +252,19 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     }
   }
   __syncthreads();
-  int lp[kRadixSteps];  // position of each item in the block's digit-ordered tile
+  int lp[STEPS];  // position of each item in the block's digit-ordered tile
 #pragma unroll
-  for (int k = 0; k < kRadixSteps; ++k) {
+  for (int k = 0; k < STEPS; ++k) {
     const int d = (key[k] >> shift) & mask;
     lp[k] = bstart[d] + wcnt[warp][d] + rank[k];
   }
   __syncthreads();  // every warp has read wcnt
   int* sk = &wcnt[0][0];
-  int* sv = sk + kRadixTile;
+  int* sv = sk + kTileOf<STEPS>;
   const int64_t left = n - tile0;
-  const int nvalid = left < kRadixTile ? (int)left : kRadixTile;
+  const int nvalid = left < kTileOf<STEPS> ? (int)left : kTileOf<STEPS>;
 #pragma unroll
-  for (int k = 0; k < kRadixSteps; ++k) {
+  for (int k = 0; k < STEPS; ++k) {
     if (wbase + k * kWarp + lane < n) {
       sk[lp[k]] = key[k];
       sv[lp[k]] = val[k];
@@ -262,7 +272,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
   }
   __syncthreads();
   const int mask_next = (1 << bits_next) - 1;
-  for (int p = threadIdx.x; p < kRadixTile; p += kRadixThreads) {
+  for (int p = threadIdx.x; p < kTileOf<STEPS>; p += kRadixThreads) {
     const bool valid = p < nvalid;
     int tag = -1 - lane;
     if (valid) {
@@ -271,13 +281,19 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
       const int64_t dst = (int64_t)hist[(int64_t)d * nblocks + blockIdx.x] + (p - bstart[d]);
       keys_out[dst] = kk;
       vals_out[dst] = sv[p];
-      tag = ((kk >> shift_next) & mask_next) * nblocks + (int)(dst / kRadixTile);
+      tag = ((kk >> shift_next) & mask_next) * nblocks + (int)(dst / kTileOf<STEPS>);
     }
     if (hist_next) {  // uniform over the launch
       const unsigned peers = __match_any_sync(0xffffffffu, tag);
       if (valid && lane == __ffs(peers) - 1) atomicAdd(&hist_next[tag], __popc(peers));
     }
   }
+}
+
+void launch_radix_scatter(int nblocks, cudaStream_t s, const int* keys_in, const int* vals_in, int* keys_out, int* vals_out,
+                          int64_t n, int shift, int bits, const int* hist) {
+  k_radix_scatter<kRadixStepsPublic><<<nblocks, kRadixThreads, 0, s>>>(keys_in, vals_in, keys_out, vals_out, n, shift, bits,
+                                                                       hist, nblocks, nullptr, 0, 0);
 }
 
 __global__ void k_gather_pos(const double* __restrict__ src, const int* __restrict__ perm, int64_t n,
@@ -372,7 +388,7 @@ __global__ void __launch_bounds__(256) k_gather_all(const double* __restrict__ s
   const int at4 = cs.n8, at1 = at4 + cs.n4;
   const int id = cell[k];
   const bool split = PHASED && __ldg(st.unordered) > st.nblocks / 2;  // uniform over the launch
-  const bool staged = st.rec && __ldg(st.staged + j / kRadixTile) != 0;
+  const bool staged = st.rec && __ldg(st.staged + j / kTileOf<kRadixSmallSteps>) != 0;
   double x, y, z;
   WordGroup<unsigned long long, 4> w8;
   WordGroup<unsigned, 4> w4;
@@ -514,41 +530,56 @@ using namespace p3m;
 // sort into tiles): fills the subtile offsets, ctx->cell (sorted ids) and
 // ctx->perm (sorted -> input index).  The first radix pass's digit histogram is
 // counted by the binning kernel and each later pass's by the scatter before it.
-static p3m_status bin_and_sort_ids(p3m_sr_ctx* ctx, const double* pos, const StageArgs& stage) {
+static p3m_status bin_and_sort_ids(p3m_sr_ctx* ctx, const double* pos, StageArgs& stage) {
   const int64_t n = ctx->n;
   cudaStream_t s = ctx->stream;
   const Geometry& g = ctx->geo;
-  p3m_status st = cuda_check(ctx, cudaMemsetAsync(ctx->offsets, 0, sizeof(int) * (g.S + 1), s), "memset offsets");
+  // the subtile counts and, in front of them, the count of unordered tiles
+  p3m_status st = cuda_check(ctx, cudaMemsetAsync(ctx->offsets - kOffsetsLead, 0, sizeof(int) * (g.S + 1 + kOffsetsLead), s),
+                             "memset offsets");
   if (st != P3M_OK) return st;
-  const int nblocks = (int)((n + kRadixTile - 1) / kRadixTile);
+  const bool small = n <= kRadixSmallN;
+  const int tile = kRadixThreads * (small ? kRadixSmallSteps : kRadixStepsPublic);
+  const int nblocks = (int)((n + tile - 1) / tile);
   int* hist[2] = {ctx->hist, ctx->hist + ctx->hist_ints};  // this pass's and the next pass's digit counts
+  const int passes = ctx->radix_passes;
+  stage.staged = ctx->staged;
+  stage.unordered = ctx->offsets - kOffsetsLead;
+  stage.nblocks = nblocks;
+  stage.drift_slots = ctx->drift_slots;
   if (n > 0) {
-    k_bin_tile<<<nblocks, kRadixThreads, 0, s>>>(pos, n, g, ctx->keys[0], ctx->vals[0], ctx->offsets, ctx->err_dev,
-                                                 hist[0], ctx->radix_bits[0], nblocks, stage);
+    auto bin = small ? k_bin_tile<kRadixSmallSteps> : k_bin_tile<kRadixStepsPublic>;
+    bin<<<nblocks, kRadixThreads, 0, s>>>(pos, n, g, ctx->keys[0], ctx->vals[0], ctx->offsets, ctx->err_dev, hist[0],
+                                          ctx->radix_bits[0], nblocks, hist[1], passes > 1 ? 1 << ctx->radix_bits[1] : 0,
+                                          stage);
     ++ctx->launches;
     if ((st = cuda_check(ctx, cudaGetLastError(), "bin kernel")) != P3M_OK) return st;
   }
-  st = cuda_check(ctx, scan_exclusive_i32(ctx->offsets, ctx->offsets, g.S + 1, ctx->scan_scratch,
-                                          ctx->scan_scratch_ints, s, &ctx->launches),
+  // the subtile offsets and the first pass's digit positions
+  st = cuda_check(ctx, scan_exclusive_i32_pair(ctx->offsets, g.S + 1, hist[0], n > 0 ? (int64_t)nblocks << ctx->radix_bits[0] : 0,
+                                               ctx->scan_scratch, ctx->scan_scratch_ints, s, &ctx->launches),
                   "scan");
   if (st != P3M_OK) return st;
   int cur = 0;
   if (n > 0) {
+    auto scatter = small ? k_radix_scatter<kRadixSmallSteps> : k_radix_scatter<kRadixStepsPublic>;
     int shift = 0;
-    for (int p = 0; p < ctx->radix_passes; ++p) {
+    for (int p = 0; p < passes; ++p) {
       const int bits = ctx->radix_bits[p];
-      const bool more = p + 1 < ctx->radix_passes;
-      st = cuda_check(ctx, scan_exclusive_i32(hist[p & 1], hist[p & 1], (int64_t)nblocks << bits, ctx->scan_scratch,
-                                              ctx->scan_scratch_ints, s,
-                                              &ctx->launches), "radix scan");
-      if (st != P3M_OK) return st;
+      const bool more = p + 1 < passes;
+      if (p > 0) {
+        st = cuda_check(ctx, scan_exclusive_i32(hist[p & 1], hist[p & 1], (int64_t)nblocks << bits, ctx->scan_scratch,
+                                                ctx->scan_scratch_ints, s, &ctx->launches), "radix scan");
+        if (st != P3M_OK) return st;
+      }
       int* next = more ? hist[(p + 1) & 1] : nullptr;
-      if (more && (st = cuda_check(ctx, cudaMemsetAsync(next, 0, sizeof(int) * ((int64_t)nblocks << ctx->radix_bits[p + 1]), s),
-                                   "memset hist")) != P3M_OK)
+      if (more && p > 0 &&  // the first pass's were cleared by the binning kernel
+          (st = cuda_check(ctx, cudaMemsetAsync(next, 0, sizeof(int) * ((int64_t)nblocks << ctx->radix_bits[p + 1]), s),
+                           "memset hist")) != P3M_OK)
         return st;
-      k_radix_scatter<<<nblocks, kRadixThreads, 0, s>>>(ctx->keys[cur], ctx->vals[cur], ctx->keys[cur ^ 1],
-                                                          ctx->vals[cur ^ 1], n, shift, bits, hist[p & 1], nblocks, next,
-                                                          shift + bits, more ? ctx->radix_bits[p + 1] : 0);
+      scatter<<<nblocks, kRadixThreads, 0, s>>>(ctx->keys[cur], ctx->vals[cur], ctx->keys[cur ^ 1], ctx->vals[cur ^ 1], n,
+                                                shift, bits, hist[p & 1], nblocks, next, shift + bits,
+                                                more ? ctx->radix_bits[p + 1] : 0);
       ++ctx->launches;
       if ((st = cuda_check(ctx, cudaGetLastError(), "radix scatter")) != P3M_OK) return st;
       cur ^= 1;
@@ -580,8 +611,8 @@ static p3m_status sort_done(p3m_sr_ctx* ctx, const double* sorted_pos) {
   ctx->sorted_pos = sorted_pos;  // the FP32 records in ctx->rel4 describe these positions
   ctx->n_drift = 0;              // no displacement since this sort
   ctx->rel4_stale = false;
-  // the drift slots and, behind them, the count of unordered tiles
-  return cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * (kMaxDrifts + 1), ctx->stream), "memset");
+  if (ctx->n > 0) return P3M_OK;  // the binning kernel cleared the drift slots
+  return cuda_check(ctx, cudaMemsetAsync(ctx->drift_slots, 0, sizeof(float) * kMaxDrifts, ctx->stream), "memset");
 }
 
 static p3m_status check_carry(p3m_sr_ctx* ctx, void* const* carry, const int* carry_bytes, int n_carry,
@@ -609,7 +640,6 @@ extern "C" p3m_status p3m_sr_sort(p3m_sr_ctx* ctx, double* pos, void* const* car
   ctx->all_chunks_built = false;
   StageArgs stage{};  // every position staged: the gather then writes them back in place
   stage.rec = (double2*)ctx->gather_tmp;
-  stage.staged = ctx->staged;
   stage.always = 1;
   if ((st = bin_and_sort_ids(ctx, pos, stage)) != P3M_OK) return st;
   if (n > 0) {
@@ -672,12 +702,9 @@ extern "C" p3m_status p3m_sr_sort_into(p3m_sr_ctx* ctx, const double* pos_in, do
   int64_t bytes = 24;
   for (int c = 0; c < n_carry; ++c) bytes += carry_bytes[c];
   if (n * bytes > kStageBytes) stage.rec = (double2*)ctx->gather_tmp;
-  stage.staged = ctx->staged;
   stage.n8 = std::min(cs.n8, 1);
   stage.n4 = stage.n8 ? 0 : std::min(cs.n4, 2);
   for (int i = 0; i < stage.n8 + stage.n4; ++i) stage.word[i] = cs.src[i];  // n8 = 0: the 4-byte arrays come first
-  stage.unordered = ctx->unordered;
-  stage.nblocks = (int)((n + kRadixTile - 1) / kRadixTile);
   const int rest = 8 * (cs.n8 - stage.n8) + 4 * (cs.n4 - stage.n4);  // one-word bytes outside the record
   stage.phased = stage.rec && 16 * n <= kStageBytes && rest >= 16;
   if ((st = bin_and_sort_ids(ctx, pos_in, stage)) != P3M_OK) return st;

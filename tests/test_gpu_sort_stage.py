@@ -56,3 +56,22 @@ def test_sort_into_matches_a_stable_cpu_sort(order, carried):
     assert torch.equal(p, q)
     for a, b in zip(arrays, out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n, x_r, n_sub", [(1, 0.2, 1), (511, 0.2, 2), (512, 0.2, 2), (513, 0.05, 1), (40_001, 0.05, 3),
+                                           (311_296, 0.03, 2), (311_297, 0.03, 2),  # the last short and the first long tile
+                                           (70_001, 0.01, 2),    # 2^23 subtiles: three radix passes
+                                           (70_001, 0.0099, 3)])  # 2.8e7 subtiles: the scans run by themselves
+def test_sort_at_the_edges_of_the_radix_tiles(n, x_r, n_sub):
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(size=(3, n))
+    perm = np.argsort(oracle.subtile_ids(pos, int(np.floor(1.0 / x_r)), n_sub), kind="stable")
+    p = torch.from_numpy(pos).cuda()
+    q, got = torch.empty_like(p), torch.empty(n, dtype=torch.int32, device="cuda")
+    with ShortRange(n, x_r / 4.5, x_r, 1.0, eps=0.01 * x_r, n_sub=n_sub) as sr:
+        for _ in range(2):  # the second finds the first one's counts in its workspaces
+            sr.sort_into(p, q, perm_out=got)
+        sr.sync()
+    order = torch.from_numpy(perm).cuda()
+    assert torch.equal(got.long(), order)
+    assert torch.equal(q, p[:, order])
