@@ -293,6 +293,14 @@ p3m_status p3m_sr_kick(p3m_sr_ctx* ctx, void* mom, int mom_precision, const void
                        const double* kick_factor);
 
 /*
+ * p3m_sr_kick of all particles with one factor, out of place: mom_out receives the kicked
+ * momenta and mom is unchanged (mom == mom_out: in place; mom NULL: zero momenta, so
+ * mom_out = a_i * kick_factor).
+ */
+p3m_status p3m_sr_kick_into(p3m_sr_ctx* ctx, const void* mom, void* mom_out, int mom_precision,
+                            const void* acc, int acc_precision, double kick_factor);
+
+/*
  * One kick of the rung-based leapfrog (Section 2.2.2, the time-stepping figure:
  * rung-l momenta are kicked every dt / 2^l, positions drift every
  * dt / 2^(n_rung-1); a particle whose rung changes jumps to a neighbouring rung
@@ -349,6 +357,13 @@ p3m_status p3m_sr_rung_kick_drift(p3m_sr_ctx* ctx, void* mom, int mom_precision,
  */
 p3m_status p3m_sr_drift(p3m_sr_ctx* ctx, double* pos, const void* mom, int mom_precision,
                         double factor);
+
+/*
+ * p3m_sr_drift out of place: pos_out (another array, not overlapping pos) receives the
+ * drifted positions and pos is unchanged.  Writing over the array of the last sort drops it.
+ */
+p3m_status p3m_sr_drift_into(p3m_sr_ctx* ctx, const double* pos, double* pos_out, const void* mom,
+                             int mom_precision, double factor);
 
 /*
  * Rungs, kick and drift in one pass over the particle arrays (Section 2.2.2:

@@ -36,6 +36,7 @@ EXPORTS = (
     "p3m_sr_permute", "p3m_sr_unpermute", "p3m_sr_forces_noalloc", "p3m_sr_forces_tabulated",
     "p3m_sr_rung_kick", "p3m_sr_set_subtiles", "p3m_sr_set_symmetric", "p3m_sr_kick_drift",
     "p3m_sr_set_count", "p3m_sr_tile_offsets", "p3m_sr_sort_into", "p3m_sr_rung_kick_drift",
+    "p3m_sr_kick_into", "p3m_sr_drift_into",
 )
 
 
@@ -84,6 +85,8 @@ def lib_path() -> str:
 def load() -> ctypes.CDLL:
     """Load libp3m_sr.so; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -115,6 +118,10 @@ def load() -> ctypes.CDLL:
         L.p3m_sr_kick.restype = i
         L.p3m_sr_drift.argtypes = [p, p, p, i, d]
         L.p3m_sr_drift.restype = i
+        L.p3m_sr_kick_into.argtypes = [p, p, p, i, p, i, d]
+        L.p3m_sr_kick_into.restype = i
+        L.p3m_sr_drift_into.argtypes = [p, p, p, p, i, d]
+        L.p3m_sr_drift_into.restype = i
         L.p3m_sr_kick_drift.argtypes = [p, p, p, i, p, i, p, d, d, d, ctypes.POINTER(d), d]
         L.p3m_sr_kick_drift.restype = i
         L.p3m_sr_vjp.argtypes = [p, p, i, p, p]
@@ -210,6 +217,16 @@ def p3m_sr_kick(ctx, mom_ptr, mom_precision, acc_ptr, acc_precision, rung_ptr, r
 def p3m_sr_drift(ctx, pos_ptr, mom_ptr, mom_precision, factor) -> int:
     return load().p3m_sr_drift(ctx, ctypes.c_void_p(pos_ptr), ctypes.c_void_p(mom_ptr), int(mom_precision),
                                float(factor))
+
+
+def p3m_sr_kick_into(ctx, mom_ptr, mom_out_ptr, mom_precision, acc_ptr, acc_precision, kick_factor) -> int:
+    return load().p3m_sr_kick_into(ctx, ctypes.c_void_p(mom_ptr or 0), ctypes.c_void_p(mom_out_ptr), int(mom_precision),
+                                   ctypes.c_void_p(acc_ptr), int(acc_precision), float(kick_factor))
+
+
+def p3m_sr_drift_into(ctx, pos_ptr, pos_out_ptr, mom_ptr, mom_precision, factor) -> int:
+    return load().p3m_sr_drift_into(ctx, ctypes.c_void_p(pos_ptr), ctypes.c_void_p(pos_out_ptr),
+                                    ctypes.c_void_p(mom_ptr), int(mom_precision), float(factor))
 
 
 def p3m_sr_kick_drift(ctx, pos_ptr, mom_ptr, mom_precision, acc_ptr, acc_precision, rung_ptr, dt, eta, eps,

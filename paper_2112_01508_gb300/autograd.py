@@ -21,15 +21,24 @@ from torch.utils.checkpoint import checkpoint
 from .shortrange import ShortRange
 
 
+def _source(t: torch.Tensor) -> torch.Tensor:
+    """t without its history, packed where its elements lie apart (the kernels need (3, n) arrays)."""
+    t = t.detach()
+    return t if t.is_contiguous() else t.clone()
+
+
 class ShortRangeAccel(torch.autograd.Function):
     """a = short-range acceleration(x) for all particles (all active)."""
 
     @staticmethod
     def forward(ctx, pos: torch.Tensor, sr: ShortRange, precision: int):
-        work = pos.detach().clone()
-        sr.sort(work)
+        src = _source(pos)
+        work = torch.empty_like(src)
+        sr.sort_into(src, work)
         sr.build_pairs()
-        acc_sorted = sr.forces(work, precision)
+        # every particle receives, so every element of the result is written
+        out = torch.empty(work.shape, dtype=torch.float32 if precision == 32 else torch.float64, device=work.device)
+        acc_sorted = sr.forces(work, precision, out=out)
         acc = sr.unpermute(acc_sorted)
         ctx.sr = sr
         ctx.precision = precision
@@ -41,8 +50,9 @@ class ShortRangeAccel(torch.autograd.Function):
         (pos,) = ctx.saved_tensors
         sr, precision = ctx.sr, ctx.precision
         dt = torch.float32 if precision == 32 else torch.float64
-        work = pos.clone()
-        sr.sort(work)  # the context may have been used since the forward
+        src = _source(pos)
+        work = torch.empty_like(src)
+        sr.sort_into(src, work)  # the context may have been used since the forward
         sr.build_pairs()
         abar_sorted = sr.permute(acc_bar.to(dt).contiguous())
         xbar_sorted = sr.vjp(work, abar_sorted, precision)
@@ -55,8 +65,9 @@ class Kick(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, mom: torch.Tensor, acc: torch.Tensor, sr: ShortRange, factor: float):
-        out = mom.detach().clone()
-        sr.kick(out, acc.detach().contiguous(), [factor])
+        src = _source(mom)
+        out = torch.empty_like(src)
+        sr.kick_into(src, out, acc.detach().contiguous(), factor)
         ctx.sr, ctx.factor = sr, factor
         ctx.acc_dtype = acc.dtype
         return out
@@ -64,8 +75,8 @@ class Kick(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gout: torch.Tensor):
         gout = gout.contiguous()
-        gacc = torch.zeros(gout.shape, dtype=ctx.acc_dtype, device=gout.device)
-        ctx.sr.kick(gacc, gout, [ctx.factor])
+        gacc = torch.empty(gout.shape, dtype=ctx.acc_dtype, device=gout.device)
+        ctx.sr.kick_into(None, gacc, gout, ctx.factor)
         return gout, gacc, None, None
 
 
@@ -74,8 +85,9 @@ class Drift(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, pos: torch.Tensor, mom: torch.Tensor, sr: ShortRange, factor: float):
-        out = pos.detach().clone()
-        sr.drift(out, mom.detach().contiguous(), factor)
+        src = _source(pos)
+        out = torch.empty_like(src)
+        sr.drift_into(src, out, mom.detach().contiguous(), factor)
         ctx.sr, ctx.factor = sr, factor
         ctx.mom_dtype = mom.dtype
         return out
@@ -83,8 +95,8 @@ class Drift(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gout: torch.Tensor):
         gout = gout.contiguous()
-        gmom = torch.zeros(gout.shape, dtype=ctx.mom_dtype, device=gout.device)
-        ctx.sr.kick(gmom, gout, [ctx.factor])
+        gmom = torch.empty(gout.shape, dtype=ctx.mom_dtype, device=gout.device)
+        ctx.sr.kick_into(None, gmom, gout, ctx.factor)
         return gout, gmom, None, None
 
 

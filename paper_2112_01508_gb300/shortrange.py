@@ -36,7 +36,7 @@ def _check(t: torch.Tensor, name: str, dtype=None, shape=None, device=None):
         raise ValueError(f"{name} must be contiguous")
     if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
         raise TypeError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     if device is not None and t.device != device:
         raise ValueError(f"{name} must be on {device}, got {t.device}")
@@ -269,6 +269,17 @@ class ShortRange:
         self._raise(nat.p3m_sr_kick(self._ctx, mom.data_ptr(), _PREC[mom.dtype], acc.data_ptr(), _PREC[acc.dtype],
                                     rung.data_ptr() if rung is not None else 0, rung_min, kf))
 
+    def kick_into(self, mom: torch.Tensor | None, out: torch.Tensor, acc: torch.Tensor, factor: float):
+        """Out-of-place kick of all particles (p3m_sr_kick_into): out = mom + factor * acc
+        (mom None: zeros)."""
+        dts = (torch.float32, torch.float64)
+        _check(out, "out", dts, (3, self.n), self.device)
+        if mom is not None:
+            _check(mom, "mom", out.dtype, (3, self.n), self.device)
+        _check(acc, "acc", dts, (3, self.n), self.device)
+        self._raise(nat.p3m_sr_kick_into(self._ctx, mom.data_ptr() if mom is not None else 0, out.data_ptr(),
+                                         _PREC[out.dtype], acc.data_ptr(), _PREC[acc.dtype], factor))
+
     def rung_kick(self, mom: torch.Tensor, acc: torch.Tensor, rung: torch.Tensor, kick_state: torch.Tensor,
                   rung_min: int, substep: int, dt: float, eta: float, eps: float, synchronize: bool = False):
         """One kick of the rung-based leapfrog with rung jumps (p3m_sr_rung_kick)."""
@@ -298,6 +309,14 @@ class ShortRange:
         _check(pos, "pos", torch.float64, (3, self.n), self.device)
         _check(mom, "mom", (torch.float32, torch.float64), (3, self.n), self.device)
         self._raise(nat.p3m_sr_drift(self._ctx, pos.data_ptr(), mom.data_ptr(), _PREC[mom.dtype], factor))
+
+    def drift_into(self, pos: torch.Tensor, out: torch.Tensor, mom: torch.Tensor, factor: float):
+        """Out-of-place drift (p3m_sr_drift_into): out = wrap(pos + factor * mom)."""
+        _check(pos, "pos", torch.float64, (3, self.n), self.device)
+        _check(out, "out", torch.float64, (3, self.n), self.device)
+        _check(mom, "mom", (torch.float32, torch.float64), (3, self.n), self.device)
+        self._raise(nat.p3m_sr_drift_into(self._ctx, pos.data_ptr(), out.data_ptr(), mom.data_ptr(), _PREC[mom.dtype],
+                                          factor))
 
     def kick_drift(self, pos: torch.Tensor, mom: torch.Tensor, acc: torch.Tensor, rung_out: torch.Tensor,
                    dt: float, eta: float, eps: float, kick_factor, drift_factor: float):

@@ -6,6 +6,8 @@ import pytest
 import torch
 
 from paper_2112_01508_gb300 import ShortRange
+from paper_2112_01508_gb300._native import P3MError
+from paper_2112_01508_gb300.autograd import Drift, Kick, short_range_accel
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +53,45 @@ def test_kick_and_drift_bits(mom_bits, acc_bits, factor):
     assert np.array_equal(out[inside].view(np.uint64), v[inside].view(np.uint64))
     assert ((out >= 0.0) & (out < 1.0)).all()
     sr.close()
+
+
+@pytest.mark.parametrize("mom_bits,acc_bits", [(32, 32), (32, 64), (64, 32), (64, 64)])
+@pytest.mark.parametrize("n", [1, 255, 5000])
+def test_out_of_place_kick_and_drift_equal_the_in_place_ones(n, mom_bits, acc_bits):
+    def bits(t):
+        return t.contiguous().view(torch.uint8)
+
+    t = {32: torch.float32, 64: torch.float64}
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.rand(3, n, generator=g, device="cuda", dtype=torch.float64)
+    q = torch.randn(3, n, generator=g, device="cuda", dtype=torch.float64).to(t[mom_bits])
+    a = torch.randn(3, n, generator=g, device="cuda", dtype=torch.float64).to(t[acc_bits])
+    with ShortRange(n, 0.02, 0.09, 1.0, eps=0.001) as sr:
+        for mom in (q, None):
+            want = q.clone() if mom is not None else torch.zeros_like(q)
+            before, out = q.clone(), torch.full_like(q, 7.0)
+            sr.kick(want, a, [0.3])
+            sr.kick_into(mom, out, a, 0.3)
+            assert torch.equal(bits(out), bits(want)) and torch.equal(q, before)
+        want, before, out = x.clone(), x.clone(), torch.full_like(x, 7.0)
+        sr.drift(want, q, 0.2)
+        sr.drift_into(x, out, q, 0.2)
+        assert torch.equal(bits(out), bits(want)) and torch.equal(x, before)
+        with pytest.raises(P3MError):
+            sr.drift_into(x, x, q, 0.2)
+        sr.sort_into(x, out)
+        sr.drift_into(x, out, q, 0.2)  # writes over the sorted positions
+        with pytest.raises(P3MError):
+            sr.build_pairs()
+
+
+def test_autograd_takes_arrays_whose_elements_lie_apart():
+    n = 500
+    g = torch.Generator(device="cuda").manual_seed(2)
+    wide = torch.rand(3, 2 * n, generator=g, device="cuda", dtype=torch.float64)
+    apart, packed = wide[:, ::2], wide[:, ::2].contiguous()
+    with ShortRange(n, 0.02, 0.09, 1.0, eps=0.001) as sr:
+        a, b = (short_range_accel(p, sr, 64) for p in (apart, packed))
+        assert torch.equal(a, b)
+        assert torch.equal(Drift.apply(apart, apart, sr, 0.1), Drift.apply(packed, packed, sr, 0.1))
+        assert torch.equal(Kick.apply(apart, packed, sr, 0.1), Kick.apply(packed, packed, sr, 0.1))
