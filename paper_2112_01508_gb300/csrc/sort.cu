@@ -104,13 +104,27 @@ __device__ __forceinline__ void stage_record(const StageArgs& st, int64_t i, con
   st.rec[2 * i + 1] = make_double2(x[2], __longlong_as_double((long long)w));
 }
 
+// One atomic per run of consecutive lanes with the same index (at: a negative one takes no
+// part).  The lanes hold nearly sorted items, whose equal indices are mostly neighbours, and a
+// shuffle and a ballot cost a fraction of __match_any_sync.
+__device__ __forceinline__ void count_runs(int* counts, int at, int lane) {
+  const int before = __shfl_up_sync(0xffffffffu, at, 1);
+  const bool head = lane == 0 || before != at;
+  const unsigned heads = __ballot_sync(0xffffffffu, head);
+  if (head && at >= 0) {
+    const unsigned after = heads & (0xfffffffeu << lane);
+    atomicAdd(&counts[at], (after ? __ffs(after) - 1 : 32) - lane);
+  }
+}
+
 // k_bin over radix tiles of kTileOf<STEPS> particles, which also counts the digits of
-// the first radix pass (bits low bits of the id) per tile: hist[d nblocks + tile].
+// the first radix pass (bits low bits of the id) per tile: hist[d nblocks + tile].  Latency
+// bound (44 us at 128^3, 31% of the issue slots); loading the next round's positions a round
+// ahead changed nothing.
 template <int STEPS>
 __global__ void __launch_bounds__(256) k_bin_tile(const double* __restrict__ pos, int64_t n, Geometry g,
-                                                  int* __restrict__ keys, int* __restrict__ vals,
-                                                  int* __restrict__ counts, int* __restrict__ err,
-                                                  int* __restrict__ hist, int bits, int nblocks,
+                                                  int* __restrict__ keys, int* __restrict__ counts,
+                                                  int* __restrict__ err, int* __restrict__ hist, int bits, int nblocks,
                                                   int* __restrict__ hist_next, int next_ints,
                                                   const __grid_constant__ StageArgs st) {
   __shared__ int cnt[1024];
@@ -133,7 +147,6 @@ __global__ void __launch_bounds__(256) k_bin_tile(const double* __restrict__ pos
       for (int d = 0; d < 3; ++d) x[d] = pos[d * n + i];
       id = bin_one(x, g, any_bad);
       keys[i] = id;
-      vals[i] = (int)i;
       atomicAdd(&cnt[id & mask], 1);
     }
     if (k == 0) {
@@ -145,8 +158,7 @@ __global__ void __launch_bounds__(256) k_bin_tile(const double* __restrict__ pos
       if (threadIdx.x == 0 && staged && st.phased) atomicAdd(st.unordered, 1);
     }
     if (staged && valid) stage_record(st, i, x);
-    const unsigned peers = __match_any_sync(0xffffffffu, valid ? id : -1 - lane);
-    if (valid && lane == __ffs(peers) - 1) atomicAdd(&counts[id], __popc(peers));
+    count_runs(counts, valid ? id : -1, lane);
   }
   if (any_bad) atomicOr(err, kErrPosition);
   __syncthreads();
@@ -172,55 +184,76 @@ __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift,
 }
 
 // Stable scatter of one radix pass.  Warp w of a block owns the contiguous
-// items [w*512, (w+1)*512) of the block's tile and walks them in 16 steps of
-// 32 consecutive items, so ranks follow the input order.  The block then puts
+// items [32 STEPS w, 32 STEPS (w + 1)) of the block's tile and walks them in STEPS rounds
+// of 32 consecutive items, so ranks follow the input order; the lanes with the same digit
+// are found by one ballot per digit bit.  The block then puts
 // its tile in digit order in shared memory and writes it out from there, so that
 // consecutive threads write consecutive positions of each digit's run.
 // hist_next (nullable, zeroed before the launch): the digit counts of the next pass
 // (bits_next bits from shift_next) per output tile, accumulated here with one atomic
-// per distinct (digit, tile) of each warp, so that pass needs no histogram kernel.
+// per run of equal (digit, tile) in a warp, so that pass needs no histogram kernel (with one,
+// a nearly sorted sort at 128^3 takes 150 us, with the atomics 138).
+// What bounds it is latency: the serial rounds and the barriers.  Counts in 16 bits, loads
+// issued before the rounds and the digits' output positions read once per block let 6 blocks
+// be resident (7 or 8 spill: 138 -> 160 us); ballots cost the same in every order, where
+// __match_any_sync took longer the more different digits a warp held.  Whole sorts before and
+// after: 15.4 M particles, nothing carried, nearly sorted 702 -> 649 us; 12 bytes carried,
+// nearly sorted 801 -> 751, in random order 1522 -> 1292; 128^3 in random order 250 -> 224.
+constexpr int kScatterBlocks = 6;
 template <int STEPS>
-__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
+__global__ void __launch_bounds__(kRadixThreads, kScatterBlocks) k_radix_scatter(
     const int* __restrict__ keys_in, const int* __restrict__ vals_in, int* __restrict__ keys_out,
     int* __restrict__ vals_out, int64_t n, int shift, int bits, const int* __restrict__ hist, int nblocks,
     int* __restrict__ hist_next, int shift_next, int bits_next) {
-  __shared__ int wcnt[kRadixWarps][kMaxRadix];  // per-warp digit counts; later the staged tile
-  __shared__ int bstart[kMaxRadix];             // first position of each digit in the block's tile
+  constexpr int kTile = kTileOf<STEPS>;
+  constexpr int kCounts = kRadixWarps * kMaxRadix * (int)sizeof(unsigned short), kStage = 2 * kTile * (int)sizeof(int);
+  __shared__ __align__(16) unsigned char area[kCounts > kStage ? kCounts : kStage];
+  unsigned short(*wcnt)[kMaxRadix] = (unsigned short(*)[kMaxRadix])area;  // per-warp digit counts (at most kTile)
+  int* sk = (int*)area;                                                   // later the staged tile
+  int* sv = sk + kTile;
+  __shared__ int bstart[kMaxRadix];  // first position of each digit in the block's tile
+  __shared__ int gstart[kMaxRadix];  // ... and its position in the output, less that
   __shared__ int wtot[kRadixWarps];
-  static_assert(kRadixWarps * kMaxRadix >= 2 * kTileOf<STEPS>, "staging area");
   const int radix = 1 << bits;
   const int mask = radix - 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int d = lane; d < radix; d += 32) wcnt[warp][d] = 0;
-  __syncwarp();
-  const int64_t tile0 = (int64_t)blockIdx.x * kTileOf<STEPS>;
+  const int64_t tile0 = (int64_t)blockIdx.x * kTile;
   const int64_t wbase = tile0 + (int64_t)warp * (STEPS * kWarp);
   const unsigned lt = (1u << lane) - 1u;
-  int key[STEPS], val[STEPS], rank[STEPS];
+  int key[STEPS], rank[STEPS];
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k) {  // all loads in flight before the serial rounds
+    const int64_t i = wbase + k * kWarp + lane;
+    key[k] = i < n ? keys_in[i] : 0;
+  }
+  for (int d = threadIdx.x; d < radix; d += kRadixThreads) gstart[d] = hist[(int64_t)d * nblocks + blockIdx.x];
+  for (int d = lane; d < radix; d += 32) wcnt[warp][d] = 0;
+  __syncwarp();
 #pragma unroll
   for (int k = 0; k < STEPS; ++k) {
-    int64_t i = wbase + k * kWarp + lane;
-    bool valid = i < n;
-    key[k] = valid ? keys_in[i] : 0;
-    val[k] = valid ? vals_in[i] : 0;
-    int d = (key[k] >> shift) & mask;
-    int tag = valid ? d : -1 - lane;  // invalid lanes match nobody
-    unsigned peers = __match_any_sync(0xffffffffu, tag);
-    int r = __popc(peers & lt);
-    int base = valid ? wcnt[warp][d] : 0;
+    const bool valid = wbase + k * kWarp + lane < n;
+    const int d = (key[k] >> shift) & mask;
+    unsigned peers = __ballot_sync(0xffffffffu, valid);  // the lanes with the same digit
+    for (int b = 0; b < bits; ++b) {
+      const bool one = (d >> b) & 1;
+      const unsigned m = __ballot_sync(0xffffffffu, one);
+      peers &= one ? m : ~m;
+    }
+    const int r = __popc(peers & lt);
+    const int base = valid ? wcnt[warp][d] : 0;
     __syncwarp();
-    if (valid && r == 0) wcnt[warp][d] = base + __popc(peers);
+    if (valid && r == 0) wcnt[warp][d] = (unsigned short)(base + __popc(peers));
     __syncwarp();
     rank[k] = base + r;
   }
   __syncthreads();
   // exclusive prefix over the warps of the block, per digit; the digit totals
-  for (int d = threadIdx.x; d < radix; d += blockDim.x) {
+  for (int d = threadIdx.x; d < radix; d += kRadixThreads) {
     int run = 0;
 #pragma unroll
     for (int w = 0; w < kRadixWarps; ++w) {
-      int t = wcnt[w][d];
-      wcnt[w][d] = run;
+      const int t = wcnt[w][d];
+      wcnt[w][d] = (unsigned short)run;
       run += t;
     }
     bstart[d] = run;
@@ -247,46 +280,49 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int d = 4 * threadIdx.x + q;
-      if (d < radix) bstart[d] = run;
+      if (d < radix) {
+        bstart[d] = run;
+        gstart[d] -= run;
+      }
       run += v[q];
     }
   }
   __syncthreads();
-  int lp[STEPS];  // position of each item in the block's digit-ordered tile
+  // position of each item in the block's digit-ordered tile
 #pragma unroll
   for (int k = 0; k < STEPS; ++k) {
     const int d = (key[k] >> shift) & mask;
-    lp[k] = bstart[d] + wcnt[warp][d] + rank[k];
+    rank[k] += bstart[d] + wcnt[warp][d];
+  }
+  int val[STEPS];
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k) {
+    const int64_t i = wbase + k * kWarp + lane;
+    val[k] = vals_in && i < n ? vals_in[i] : (int)i;  // first pass: the values are the positions
   }
   __syncthreads();  // every warp has read wcnt
-  int* sk = &wcnt[0][0];
-  int* sv = sk + kTileOf<STEPS>;
   const int64_t left = n - tile0;
-  const int nvalid = left < kTileOf<STEPS> ? (int)left : kTileOf<STEPS>;
+  const int nvalid = left < kTile ? (int)left : kTile;
 #pragma unroll
   for (int k = 0; k < STEPS; ++k) {
     if (wbase + k * kWarp + lane < n) {
-      sk[lp[k]] = key[k];
-      sv[lp[k]] = val[k];
+      sk[rank[k]] = key[k];
+      sv[rank[k]] = val[k];
     }
   }
   __syncthreads();
   const int mask_next = (1 << bits_next) - 1;
-  for (int p = threadIdx.x; p < kTileOf<STEPS>; p += kRadixThreads) {
+  for (int p = threadIdx.x; p < kTile; p += kRadixThreads) {
     const bool valid = p < nvalid;
-    int tag = -1 - lane;
+    int tag = -1;
     if (valid) {
       const int kk = sk[p];
-      const int d = (kk >> shift) & mask;
-      const int64_t dst = (int64_t)hist[(int64_t)d * nblocks + blockIdx.x] + (p - bstart[d]);
+      const int dst = gstart[(kk >> shift) & mask] + p;  // n < 2^31 - 64
       keys_out[dst] = kk;
       vals_out[dst] = sv[p];
-      tag = ((kk >> shift_next) & mask_next) * nblocks + (int)(dst / kTileOf<STEPS>);
+      tag = ((kk >> shift_next) & mask_next) * nblocks + (int)((unsigned)dst / kTile);
     }
-    if (hist_next) {  // uniform over the launch
-      const unsigned peers = __match_any_sync(0xffffffffu, tag);
-      if (valid && lane == __ffs(peers) - 1) atomicAdd(&hist_next[tag], __popc(peers));
-    }
+    if (hist_next) count_runs(hist_next, tag, lane);  // uniform over the launch
   }
 }
 
@@ -549,7 +585,7 @@ static p3m_status bin_and_sort_ids(p3m_sr_ctx* ctx, const double* pos, StageArgs
   stage.drift_slots = ctx->drift_slots;
   if (n > 0) {
     auto bin = small ? k_bin_tile<kRadixSmallSteps> : k_bin_tile<kRadixStepsPublic>;
-    bin<<<nblocks, kRadixThreads, 0, s>>>(pos, n, g, ctx->keys[0], ctx->vals[0], ctx->offsets, ctx->err_dev, hist[0],
+    bin<<<nblocks, kRadixThreads, 0, s>>>(pos, n, g, ctx->keys[0], ctx->offsets, ctx->err_dev, hist[0],
                                           ctx->radix_bits[0], nblocks, hist[1], passes > 1 ? 1 << ctx->radix_bits[1] : 0,
                                           stage);
     ++ctx->launches;
@@ -573,13 +609,13 @@ static p3m_status bin_and_sort_ids(p3m_sr_ctx* ctx, const double* pos, StageArgs
         if (st != P3M_OK) return st;
       }
       int* next = more ? hist[(p + 1) & 1] : nullptr;
-      if (more && p > 0 &&  // the first pass's were cleared by the binning kernel
+      if (more && p > 0 &&  // the second pass's were cleared by the binning kernel
           (st = cuda_check(ctx, cudaMemsetAsync(next, 0, sizeof(int) * ((int64_t)nblocks << ctx->radix_bits[p + 1]), s),
                            "memset hist")) != P3M_OK)
         return st;
-      scatter<<<nblocks, kRadixThreads, 0, s>>>(ctx->keys[cur], ctx->vals[cur], ctx->keys[cur ^ 1], ctx->vals[cur ^ 1], n,
-                                                shift, bits, hist[p & 1], nblocks, next, shift + bits,
-                                                more ? ctx->radix_bits[p + 1] : 0);
+      scatter<<<nblocks, kRadixThreads, 0, s>>>(ctx->keys[cur], p > 0 ? ctx->vals[cur] : nullptr, ctx->keys[cur ^ 1],
+                                                ctx->vals[cur ^ 1], n, shift, bits, hist[p & 1], nblocks, next,
+                                                shift + bits, more ? ctx->radix_bits[p + 1] : 0);
       ++ctx->launches;
       if ((st = cuda_check(ctx, cudaGetLastError(), "radix scatter")) != P3M_OK) return st;
       cur ^= 1;
