@@ -97,7 +97,7 @@ def hbm_peak():
 
 
 FORCE_SOURCES = ["paper_2112_01508_gb300/csrc/force.cu", "paper_2112_01508_gb300/csrc/pair_math.cuh",
-                 "paper_2112_01508_gb300/csrc/common.cuh"]
+                 "paper_2112_01508_gb300/csrc/traverse.cuh", "paper_2112_01508_gb300/csrc/common.cuh"]
 
 
 class ClockSampler:

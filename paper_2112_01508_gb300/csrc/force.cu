@@ -1,5 +1,5 @@
-// Receiver work lists, the short-range pair-force kernels (FP32 and FP64) and
-// the adjoint (VJP) kernels.
+// Receiver work lists, the FP32 short-range pair-force kernels and their adjoints
+// (VJP); the FP64 ones are in pair64.cu, and the traversal they share in traverse.cuh.
 //
 // Paper design (Section 2.1.3): tiles of side >= x_r, subtiles inside them,
 // precomputed subtile pairings inside a "blocky ball" of radius x_r, a
@@ -20,13 +20,11 @@
 //   3. walks the concatenated supplier ranges 32 at a time: each lane loads
 //      one supplier j (FP32 coordinates relative to its subtile origin, moved
 //      into the chunk frame by the integer subtile offset) and tests it against
-//      the bounding box; the survivors are broadcast to all lanes, and every
-//      lane evaluates its own (i, j) pair.
-// The one-sided FP32 forward kernel stages the survivors in shared memory as
-// packed pairs and evaluates two suppliers per step in f32x2 arithmetic; the
-// FP64 forward and the one-sided adjoint broadcast survivors with warp
-// shuffles.  With every particle a receiver, the FP32 forward and the FP32
-// adjoint evaluate each pair once instead (k_force_sym, below).  Chunks are
+//      the bounding box.
+// The one-sided kernels stage the survivors in shared memory as packed pairs,
+// and every lane evaluates its own receiver with two suppliers per step in f32x2
+// arithmetic.  With every particle a receiver, the forward and the adjoint
+// evaluate each pair once instead (k_force_sym, below).  Chunks are
 // handed out through an atomic counter to persistent warps, which balances the
 // strongly varying cost of clustered regions.
 #include <algorithm>
@@ -316,9 +314,8 @@ __device__ __forceinline__ void store_result(const TraversalArgs& a, const Chunk
 }
 
 // ---------------------------------------------------------------------------
-// FP32 forward, packed broadcast variant: the structure of the generic kernel
-// (32 receivers per warp, every surviving supplier tested by all lanes), but
-// the survivors of a batch are staged, compacted and negated, in shared memory
+// FP32 forward, one-sided: 32 receivers per warp, every surviving supplier tested
+// by all lanes; the survivors of a batch are staged, compacted and negated, in shared memory
 // as packed pairs, read back with broadcast loads, and two suppliers are
 // evaluated per step in f32x2 arithmetic.
 // ---------------------------------------------------------------------------

@@ -5,8 +5,8 @@
 // GPU design: one pass bins every particle (subtile id from one correctly
 // rounded multiply per dimension) and builds the subtile histogram; an
 // exclusive scan turns it into the subtile offsets.  The permutation itself
-// comes from a stable LSD radix sort of the subtile ids (8-bit digits at
-// most, warp-level ranking with match.any so that equal ids keep their input
+// comes from a stable LSD radix sort of the subtile ids (digits of at most
+// 10 bits, warp-level ranking with ballots so that equal ids keep their input
 // order), after which positions and any carried arrays are gathered.
 #include <algorithm>
 #include <string>
