@@ -31,3 +31,31 @@ def test_assignment_and_accel(n_phi, p_i):
             assert _rel(lr.assign(dev).cpu().numpy().astype(np.float64), rho) <= tol_rho
             assert _rel(lr.accel(dev).cpu().numpy().astype(np.float64), acc) <= tol_acc
             lr.sync()
+
+
+@pytest.mark.parametrize("p_i", [1, 2, 3, 4])
+@pytest.mark.parametrize("n_phi,box", [(8, 1.0), (30, 3.0), (256, 0.7)])
+def test_positions_at_cell_faces_and_centres(n_phi, box, p_i):
+    # faces and centres of cells and their neighbours in double, both zeros, tiny and the last
+    # positions of the box: the cell and the offset come from the bit patterns
+    k = np.arange(n_phi + 1)
+    at = np.concatenate([k * (box / n_phi), (k[:-1] + 0.5) * (box / n_phi)])
+    x = np.concatenate([at, np.nextafter(at, -1.0), np.nextafter(at, 9.0), [0.0, -0.0, 5e-324, 1e-300, 1e-17, np.nextafter(box, 0)]])
+    x = x[(x >= 0.0) & (x < box)]
+    rng = np.random.default_rng(p_i)
+    pos = np.stack([x, rng.permutation(x), rng.permutation(x)])
+    dev = torch.from_numpy(pos).cuda()
+    n = pos.shape[1]
+    rho = opm.assign(pos / box, n_phi, p_i) if box == 1.0 else None
+    fx = np.floor(pos * (n_phi / box) - 0.5 + (0.5 if p_i % 2 else 0.0))  # a cell is the oracle's or its neighbour with weight 0
+    for precision, tol in ((32, 1e-6), (64, 1e-14)):
+        with LongRange(n, n_phi, 1.25 * box / n_phi, 1.0 / n, p_i=p_i, p_d=4, precision=precision, box=box) as lr:
+            got = lr.assign(dev).cpu().numpy().astype(np.float64)
+            lr.sync()
+        assert abs(got.sum() - n) <= tol * n
+        if rho is not None:
+            assert _rel(got, rho) <= tol
+        if p_i == 1:
+            want = np.zeros((n_phi,) * 3)
+            np.add.at(want, tuple(fx.astype(int) % n_phi), 1.0)
+            assert np.array_equal(got, want)
