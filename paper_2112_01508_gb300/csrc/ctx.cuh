@@ -72,7 +72,7 @@ struct p3m_sr_ctx {
   const double* sorted_pos = nullptr;  // array sorted by the last p3m_sr_sort (rel4 matches it)
   float* drift_slots = nullptr;        // kMaxDrifts: largest displacement of each drift since the sort
   int n_drift = 0;                     // drifts applied to sorted_pos since the sort
-  bool rel4_stale = false;             // sorted_pos moved after rel4 was written
+  bool rel4_stale = false;             // rel4 is not of sorted_pos as it is now (it moved, or another array's was built)
   bool pairs_built = false;
   bool all_chunks_built = false;
   bool all_active = true;

@@ -1313,12 +1313,15 @@ static p3m_status clear_counters(p3m_sr_ctx* ctx) {
   return cuda_check(ctx, cudaMemsetAsync(ctx->dev_small + 3, 0, 5 * sizeof(int), ctx->stream), "memset");
 }
 
+// Records of pos.  ctx->rel4 holds those of sorted_pos unless rel4_stale says otherwise, so
+// building another array's leaves it stale: every pair kernel, the FP64 ones included, finds
+// its candidates from these records.
 static p3m_status prepare_rel4(p3m_sr_ctx* ctx, const double* pos) {
   if (ctx->n == 0) return P3M_OK;
-  if (pos == ctx->sorted_pos && !ctx->rel4_stale) return P3M_OK;  // written by the sort for these positions
+  if (pos == ctx->sorted_pos && !ctx->rel4_stale) return P3M_OK;  // written by the sort or an earlier call
   k_rel4<<<blocks_for(ctx->n, 256), 256, 0, ctx->stream>>>(pos, ctx->cell, ctx->n, ctx->geo, ctx->rel4);
   ++ctx->launches;
-  if (pos == ctx->sorted_pos) ctx->rel4_stale = false;
+  ctx->rel4_stale = pos != ctx->sorted_pos;
   return cuda_check(ctx, cudaGetLastError(), "rel4 kernel");
 }
 
