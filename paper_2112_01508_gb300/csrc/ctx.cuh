@@ -96,6 +96,9 @@ p3m_status ensure_all_chunks(p3m_sr_ctx* ctx);
 // The FP64 kernels' tables (pair64.cu): their size, and filling ctx->tab64 on the stream.
 int64_t pair_table_doubles();
 p3m_status fill_pair_tables(p3m_sr_ctx* ctx);
+// Power of two by which the FP32 records that the FP64 kernels read are scaled (1 unless the box
+// is beyond the range of floats).
+double rel_unit(double box);
 // FP64 forces or adjoint on the chunks of `a`.
 struct TraversalArgs;
 cudaError_t launch_pair64(p3m_sr_ctx* ctx, const TraversalArgs& a, bool vjp);

@@ -55,7 +55,9 @@ static unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 
 // FP32 coordinates relative to the particle's subtile origin, plus the id bits.
 // All lanes of a warp reach the vote: launched with whole warps, lanes past n only vote.
-__global__ void k_rel4(const double* __restrict__ pos, const int* __restrict__ cell, int64_t n, Geometry g,
+// SCALED: times `scale`, a power of two (FP64 pairs of a box beyond the range of floats).
+template <bool SCALED>
+__global__ void k_rel4(const double* __restrict__ pos, const int* __restrict__ cell, int64_t n, Geometry g, double scale,
                        float4* __restrict__ rel4) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = i < n;
@@ -70,6 +72,11 @@ __global__ void k_rel4(const double* __restrict__ pos, const int* __restrict__ c
   }
   double r[3];
   rel_to_subtile(g, x, y, z, gx, gy, gz, r);
+  if constexpr (SCALED) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r[d] *= scale;
+    g.box *= scale;
+  }
   float f[3] = {narrow(r[0]), narrow(r[1]), narrow(r[2])};
   // relative to the origin of the subtile of the last sort; a particle that drifted
   // across the periodic boundary since then takes its nearest image.  Its offset is
@@ -1301,6 +1308,7 @@ static TraversalArgs base_args(p3m_sr_ctx* ctx) {
   a.n = ctx->n;
   a.rel4 = ctx->rel4;
   a.rel_scale = 1.0f;
+  a.unit = 1.0;
   a.pairs = ctx->pair_count;
   a.drift_slots = ctx->drift_slots;
   a.n_drift = ctx->n_drift;
@@ -1316,12 +1324,16 @@ static p3m_status clear_counters(p3m_sr_ctx* ctx) {
 // Records of pos.  ctx->rel4 holds those of sorted_pos unless rel4_stale says otherwise, so
 // building another array's leaves it stale: every pair kernel, the FP64 ones included, finds
 // its candidates from these records.
-static p3m_status prepare_rel4(p3m_sr_ctx* ctx, const double* pos) {
+// For the FP64 kernels of a box whose records would leave the range of floats (rel_unit) they
+// are built in its units, each time: for other calls they are stale too.
+static p3m_status prepare_rel4(p3m_sr_ctx* ctx, const double* pos, int precision) {
   if (ctx->n == 0) return P3M_OK;
-  if (pos == ctx->sorted_pos && !ctx->rel4_stale) return P3M_OK;  // written by the sort or an earlier call
-  k_rel4<<<blocks_for(ctx->n, 256), 256, 0, ctx->stream>>>(pos, ctx->cell, ctx->n, ctx->geo, ctx->rel4);
+  const double unit = precision == 64 ? rel_unit(ctx->prm.box) : 1.0;
+  if (unit == 1.0 && pos == ctx->sorted_pos && !ctx->rel4_stale) return P3M_OK;  // written by the sort or an earlier call
+  auto kernel = unit == 1.0 ? k_rel4<false> : k_rel4<true>;
+  kernel<<<blocks_for(ctx->n, 256), 256, 0, ctx->stream>>>(pos, ctx->cell, ctx->n, ctx->geo, unit, ctx->rel4);
   ++ctx->launches;
-  ctx->rel4_stale = pos != ctx->sorted_pos;
+  ctx->rel4_stale = unit != 1.0 || pos != ctx->sorted_pos;
   return cuda_check(ctx, cudaGetLastError(), "rel4 kernel");
 }
 
@@ -1373,7 +1385,7 @@ extern "C" p3m_status p3m_sr_forces(p3m_sr_ctx* ctx, const double* pos, int prec
   cudaStream_t s = ctx->stream;
   if ((st = clear_counters(ctx)) != P3M_OK) return st;
   if (ctx->n == 0) return P3M_OK;
-  if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
+  if ((st = prepare_rel4(ctx, pos, precision)) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
   a.chunks = ctx->chunks;
@@ -1449,7 +1461,7 @@ extern "C" p3m_status p3m_sr_forces_tabulated(p3m_sr_ctx* ctx, const double* pos
   }
   if ((st = clear_counters(ctx)) != P3M_OK) return st;
   if (ctx->n == 0) return P3M_OK;
-  if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
+  if ((st = prepare_rel4(ctx, pos, 32)) != P3M_OK) return st;
   TraversalArgs a = base_args(ctx);
   a.pos = pos;
   a.chunks = ctx->chunks;
@@ -1510,7 +1522,7 @@ extern "C" p3m_status p3m_sr_vjp(p3m_sr_ctx* ctx, const double* pos, int precisi
       return st;
   }
   if ((st = ensure_all_chunks(ctx)) != P3M_OK) return st;
-  if ((st = prepare_rel4(ctx, pos)) != P3M_OK) return st;
+  if ((st = prepare_rel4(ctx, pos, precision)) != P3M_OK) return st;
   if (precision == 32)
     k_abar_f32<<<blocks_for(n, 256), 256, 0, s>>>((const float*)acc_bar, ctx->active_flag, ctx->all_active, n,
                                                    ctx->abar4);
@@ -1747,6 +1759,7 @@ extern "C" p3m_status p3m_sr_forces_noalloc(const p3m_sr_params* params, void* c
   a.pos = spos;
   a.rel4 = rel4;
   a.rel_scale = 1.0f;
+  a.unit = 1.0;
   a.offsets = offsets;
   a.chunks = chunks;
   a.n_chunks = small + 0;

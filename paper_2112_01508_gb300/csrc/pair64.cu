@@ -534,6 +534,13 @@ __global__ void k_parts_finish64(TraversalArgs a, double scale) {
   }
 }
 
+// The FP32 records are in the units of the positions where those fit a float with room for
+// a product with 2^-26, which is nearly always; else in units of the box's binary exponent.
+double rel_unit(double box) {
+  const int k = std::ilogb(box);
+  return k >= -100 && k <= 120 ? 1.0 : std::ldexp(1.0, -k);
+}
+
 static Pair64Args pair64_args(const p3m_sr_ctx* ctx) {
   const p3m_sr_params& q = ctx->prm;
   const ForceConsts& f = ctx->fc;
@@ -608,7 +615,8 @@ static cudaError_t launch_pair64_soft(p3m_sr_ctx* ctx, TraversalArgs a) {
   cudaError_t e = cudaFuncSetAttribute(k_pair64<VJP, SOFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxShared);
   if (e != cudaSuccess) return e;
   const int slot = VJP ? 1 : 0;
-  a.rel_scale = (float)p.len;
+  a.unit = p.len;
+  a.rel_scale = rel_unit(ctx->prm.box) == 1.0 ? (float)p.len : 1.0f;
   for (int d = 0; d < 3; ++d) a.g.side32[d] = (float)(a.g.side64[d] * p.len);
   a.f.margin2_f = (float)(p.len * p.len * (ctx->prm.x_r * ctx->prm.x_r * (1.0 + 1e-4)));
   a.part_acc = ctx->part_acc;

@@ -18,6 +18,7 @@ struct TraversalArgs {
   const double* pos;          // FP64 path positions
   const float4* rel4;         // FP32 coordinates relative to the subtile, and its id
   float rel_scale;            // power of two that brings rel4 into the units of g.side32 and f.margin2_f
+  double unit;                // the same for lengths
   const int* offsets;         // S + 1 subtile offsets
   const Chunk* chunks;
   float4* part_acc;           // per (work item, lane) partial sums when chunks are split, or nullptr
@@ -98,17 +99,17 @@ __device__ __forceinline__ Reach make_reach(const TraversalArgs& a) {
     r.delta = 0.0f;
     return r;
   }
-  r.delta = delta * a.rel_scale;
-  const double dl = (double)delta * (1.0 + 1e-5) * a.rel_scale;  // the float sum may round down
+  r.delta = (float)(delta * a.unit);
+  const double dl = (double)delta * (1.0 + 1e-5) * a.unit;  // the float sum may round down
   const double reach = sqrt((double)a.f.margin2_f) + dl;
-  const double half = 0.5 * a.g.box * a.rel_scale;
-  if (!(reach + dl < half)) {
+  const double half = 0.5 * a.g.box * a.unit;
+  if (!(reach + dl < half) || delta >= 3.0e38f) {  // (the bound of a drift saturates there)
     if ((threadIdx.x & 31) == 0 && a.err) atomicOr(a.err, kErrDrift);
   }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const double rr = fmin(reach + dl, half);
-    r.R[d] = (int)ceil(rr / (a.g.side64[d] * a.rel_scale) * (1.0 + 1e-12));
+    r.R[d] = (int)ceil(rr / (a.g.side64[d] * a.unit) * (1.0 + 1e-12));
   }
   r.sub2 = (float)(reach * reach * (1.0 + 1e-6));
   return r;
