@@ -27,14 +27,22 @@ def _source(t: torch.Tensor) -> torch.Tensor:
     return t if t.is_contiguous() else t.clone()
 
 
+def _sorted_copy(pos: torch.Tensor, sr: ShortRange) -> torch.Tensor:
+    """pos in the sorted order.  The context refers to the copy until the next sort, so it lives
+    that long: its memory must not come back as another tensor's that a drift writes to."""
+    src = _source(pos)
+    work = torch.empty_like(src)
+    sr.sort_into(src, work)
+    sr._sorted = work
+    return work
+
+
 class ShortRangeAccel(torch.autograd.Function):
     """a = short-range acceleration(x) for all particles (all active)."""
 
     @staticmethod
     def forward(ctx, pos: torch.Tensor, sr: ShortRange, precision: int):
-        src = _source(pos)
-        work = torch.empty_like(src)
-        sr.sort_into(src, work)
+        work = _sorted_copy(pos, sr)
         sr.build_pairs()
         # every particle receives, so every element of the result is written
         out = torch.empty(work.shape, dtype=torch.float32 if precision == 32 else torch.float64, device=work.device)
@@ -50,9 +58,7 @@ class ShortRangeAccel(torch.autograd.Function):
         (pos,) = ctx.saved_tensors
         sr, precision = ctx.sr, ctx.precision
         dt = torch.float32 if precision == 32 else torch.float64
-        src = _source(pos)
-        work = torch.empty_like(src)
-        sr.sort_into(src, work)  # the context may have been used since the forward
+        work = _sorted_copy(pos, sr)  # the context may have been used since the forward
         sr.build_pairs()
         abar_sorted = sr.permute(acc_bar.to(dt).contiguous())
         xbar_sorted = sr.vjp(work, abar_sorted, precision)

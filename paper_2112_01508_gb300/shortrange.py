@@ -78,6 +78,7 @@ class ShortRange:
         if st != nat.P3M_OK:
             raise nat.P3MError(st, "p3m_sr_create failed (check parameters / device memory)")
         self._ctx = ctx
+        self._sorted = None  # a sorted array that nobody else holds (the autograd functions')
         self.set_symmetric(symmetric)
 
     @classmethod
@@ -92,6 +93,7 @@ class ShortRange:
         if getattr(self, "_ctx", None):
             nat.p3m_sr_destroy(self._ctx)
             self._ctx = None
+            self._sorted = None
 
     def __del__(self):
         try:
@@ -185,6 +187,7 @@ class ShortRange:
                              perm_out.data_ptr() if perm_out is not None else 0,
                              subtile_id_out.data_ptr() if subtile_id_out is not None else 0)
         self._raise(st)
+        self._sorted = None
 
     def _carry_ptrs(self, carry, name):
         ptrs, nbytes = [], []
@@ -222,6 +225,7 @@ class ShortRange:
         self._raise(nat.p3m_sr_sort_into(self._ctx, pos.data_ptr(), pos_out.data_ptr(), pin, pout, nb,
                                          perm_out.data_ptr() if perm_out is not None else 0,
                                          subtile_id_out.data_ptr() if subtile_id_out is not None else 0))
+        self._sorted = None
 
     def build_pairs(self, rung: torch.Tensor | None = None, rung_min: int = 0):
         if rung is not None:
