@@ -111,20 +111,12 @@ __device__ __forceinline__ int quot_small(int a, int b, float inv) {
   return q;
 }
 
-// encode_subtile for 0 <= g < M with the quotients by n_sub from quot_small.
+// Id of subtile (gx, gy, gz), 0 <= g < M, with the quotients by n_sub from quot_small.
 __device__ __forceinline__ int encode_subtile_fast(const Geometry& g, int gx, int gy, int gz) {
   const int tx = quot_small(gx, g.ns[0], g.inv_ns[0]), sx = gx - tx * g.ns[0];
   const int ty = quot_small(gy, g.ns[1], g.inv_ns[1]), sy = gy - ty * g.ns[1];
   const int tz = quot_small(gz, g.ns[2], g.inv_ns[2]), sz = gz - tz * g.ns[2];
   const int tile = (tx * g.n_t + ty) * g.n_t + tz;
-  return tile * g.nsub3 + (sx * g.ns[1] + sy) * g.ns[2] + sz;
-}
-
-__device__ __forceinline__ int encode_subtile(const Geometry& g, int gx, int gy, int gz) {
-  int tx = gx / g.ns[0], sx = gx - tx * g.ns[0];
-  int ty = gy / g.ns[1], sy = gy - ty * g.ns[1];
-  int tz = gz / g.ns[2], sz = gz - tz * g.ns[2];
-  int tile = (tx * g.n_t + ty) * g.n_t + tz;
   return tile * g.nsub3 + (sx * g.ns[1] + sy) * g.ns[2] + sz;
 }
 
@@ -186,8 +178,6 @@ __global__ void k_bin(const double* __restrict__ pos, int64_t n, Geometry g, int
                       int* __restrict__ vals, int* __restrict__ counts, int* __restrict__ err);
 __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift, int bits, int* __restrict__ hist,
                              int nblocks);
-__global__ void k_gather_pos(const double* __restrict__ src, const int* __restrict__ perm, int64_t n,
-                             double* __restrict__ dst);
 
 // ---- launch helpers (host) --------------------------------------------------
 

@@ -340,12 +340,6 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   return d;
 }
 
-// cp.async record copies as in k_force_sym (2.087 -> 2.052 ms all active on the
-// 128^3 set).
-#ifndef P3M_GP_CPASYNC
-#define P3M_GP_CPASYNC 1
-#endif
-
 // Survivors staged before they are evaluated: more than one batch of 32, so that the loop is
 // entered, and its last pair padded, half as often (against 32: 2 M particles all active 1.794
 // -> 1.773 ms, a third 0.917 -> 0.907, tabulated 1.474 -> 1.432; 96: no more).
@@ -354,17 +348,12 @@ struct PackedSmem {
   WarpList L;
   float4 sxy[kGpStage / 2 + 1];  // (-xa, -xb, -ya, -yb)
   float2 sz[kGpStage / 2 + 1];   // (-za, -zb)
-#if P3M_GP_CPASYNC
-  float4 rec[2][kWarp];       // records of the current and the next batch
-#endif
+  float4 rec[2][kWarp];          // records of the current and the next batch, by cp.async as in k_force_sym
 };
 
 // 7 resident blocks of 4 warps per SM bound the kernel to 70 registers (no
 // spills); with the cp.async staging measured best among 5 to 8 on the state of the
 // 128^3 set after 25 benchmark steps (deep-rung substep 3% faster than with 6).
-#ifndef P3M_GP_SOFT2
-#define P3M_GP_SOFT2 1  // close pairs of both halves in one packed softened evaluation
-#endif
 #ifndef P3M_GP_UNROLL
 #define P3M_GP_UNROLL 2  // supplier pairs per loop iteration (2: 2-3% faster than 1 on the 128^3 set)
 #endif
@@ -449,16 +438,9 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
                 const bool rare0 = h0 && (q0 < a.f.rsw2_f) && (q0 > kR2Self);
                 const bool rare1 = h1 && (q1 < a.f.rsw2_f) && (q1 > kR2Self);
                 if (__any_sync(full, rare0 || rare1)) {
-#if P3M_GP_SOFT2
                   float b0, b1, s0, s1;
                   upk(B, b0, b1);
                   upk(bracket_soft_f32x2<SOFT>(r2, a.f, a.sc), s0, s1);
-#else
-                  float b0, b1, Ds;
-                  upk(B, b0, b1);
-                  const float s0 = bracket_soft_f32<SOFT, false>(q0, a.f, a.sc, Ds);
-                  const float s1 = bracket_soft_f32<SOFT, false>(q1, a.f, a.sc, Ds);
-#endif
                   if (rare0) b0 = s0;
                   if (rare1) b1 = s1;
                   B = pk(b0, b1);
@@ -486,27 +468,18 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_force_packed(Tr
       int jn;
       unsigned dn;
       bool vn = locate(0, jn, dn);
-#if P3M_GP_CPASYNC
       int buf = 0;
       if (vn) cp_async16(&S.rec[0][lane], a.rel4 + jn);
       cp_async_commit();
-#else
-      float4 rn = vn ? a.rel4[jn] : make_float4(0.f, 0.f, 0.f, 0.f);
-#endif
       for (int b = 0; b < total; b += kWarp) {
         const bool have = vn;
         const unsigned dpk = dn;
         vn = (b + kWarp < total) ? locate(b + kWarp, jn, dn) : false;
-#if P3M_GP_CPASYNC
         if (vn) cp_async16(&S.rec[buf ^ 1][lane], a.rel4 + jn);
         cp_async_commit();
         cp_async_wait_prev();  // this lane's copy of batch b has landed
         const float4 r = have ? S.rec[buf][lane] : make_float4(0.f, 0.f, 0.f, 0.f);
         buf ^= 1;
-#else
-        const float4 r = rn;
-        if (vn) rn = a.rel4[jn];
-#endif
         bool keep = false, near = false;
         Vec3<float> pj = {0.f, 0.f, 0.f};
         if (have) {
@@ -1138,16 +1111,10 @@ __global__ void __launch_bounds__(kPThreads, P3M_GP_MINBLOCKS) k_vjp_packed(Trav
             if (kCheckSoft) {
               const bool rare0 = h0 && (q0 < a.f.rsw2_f), rare1 = h1 && (q1 < a.f.rsw2_f);
               if (__any_sync(full, rare0 || rare1)) {
-#if P3M_GP_SOFT2
                 f2 Dsp;
                 float s0, s1, Ds0, Ds1;
                 upk(bracket_soft_vjp_f32x2<SOFT>(r2, a.f, a.sc, Dsp), s0, s1);
                 upk(Dsp, Ds0, Ds1);
-#else
-                float Ds0, Ds1;
-                const float s0 = bracket_soft_f32<SOFT, true>(q0, a.f, a.sc, Ds0);
-                const float s1 = bracket_soft_f32<SOFT, true>(q1, a.f, a.sc, Ds1);
-#endif
                 if (rare0) { b0 = s0; d0 = Ds0; }
                 if (rare1) { b1 = s1; d1 = Ds1; }
               }

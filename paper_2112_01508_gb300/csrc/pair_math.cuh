@@ -75,38 +75,8 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
 
 // ---------------------------------------------------------------- FP32 ----
 
-// Main branch.  Returns B; with VJP also D = B'(r)/r.
-template <int SOFT, bool VJP>
-__device__ __forceinline__ float bracket_main_f32(float r2, const ForceConsts& f, float& D) {
-  float rinv = rsqrt_approx(r2);
-  float r = r2 * rinv;
-  float e = ex2_approx(r2 * f.ce_f);
-  float t = rcp_approx(fmaf(r, f.kc_f, 1.0f));
-  float q = fmaf(f.c_f[5], t, f.c_f[4]);
-  q = fmaf(q, t, f.c_f[3]);
-  q = fmaf(q, t, f.c_f[2]);
-  q = fmaf(q, t, f.c_f[1]);
-  q = fmaf(q, t, f.c_f[0]);
-  float ex = q * t;  // erfcx(u)
-  float rinv2 = rinv * rinv;
-  float er2 = e * rinv2;
-  float B = er2 * fmaf(ex, rinv, f.k2_f);
-  if (VJP) {
-    // g'(r)/r = -r^{-2} (3 g + exp(-u^2) / (2 sqrt(pi) x_s^3))
-    D = -rinv2 * fmaf(3.0f, B, e * f.k3_f);
-  }
-  if (SOFT == P3M_SOFT_PLUMMER) {
-    float p = rsqrt_approx(r2 + f.eps2_f);
-    float p3 = p * p * p;
-    float rinv3 = rinv2 * rinv;
-    if (VJP) D += 3.0f * (rinv3 * rinv2 - p3 * p * p);
-    B += p3 - rinv3;
-  }
-  return B;
-}
-
-// Main branch for two pairs at once (forward only): the FP32 chain of
-// bracket_main_f32 in packed f32x2 form; the SFU operations stay scalar.
+// Main branch for two pairs at once (forward only): the FP32 chain in packed f32x2
+// form; the SFU operations stay scalar.
 template <int SOFT>
 __device__ __forceinline__ f2 bracket_main_f32x2(f2 r2, const ForceConsts& f) {
   float a, b;
@@ -176,49 +146,6 @@ __device__ __forceinline__ f2 bracket_main_vjp_f32x2(f2 r2, const ForceConsts& f
     B = add2(B, fma2(rinv3, pk(-1.0f, -1.0f), p3));
   }
   return B;
-}
-
-// Softened branch, r^2 < r_sw^2 (and r = 0 for point particles).
-template <int SOFT, bool VJP>
-__device__ __forceinline__ float bracket_soft_f32(float r2, const ForceConsts& f, const SeriesConsts& sc,
-                                                  float& D) {
-  if (SOFT == P3M_SOFT_NONE) {  // only coincident particles arrive here: zero by convention
-    D = 0.0f;
-    return 0.0f;
-  }
-  float r = sqrtf(r2);
-  float u = r * f.inv2xs_f;
-  float u2 = u * u;
-  float h = sc.h_f[kHTermsF - 1];
-#pragma unroll
-  for (int k = kHTermsF - 2; k >= 0; --k) h = fmaf(h, u2, sc.h_f[k]);
-  float s3, ds;  // |x|^{-3}_shape and its r-derivative divided by r
-  if (SOFT == P3M_SOFT_BSPLINE) {
-    float x = r * f.inv_epsb_f;
-    float c = f.bnorm_f;
-    float ce = c * f.inv_epsb_f * f.inv_epsb_f;  // 32 / eps_B^5
-    if (x < 0.5f) {
-      s3 = c * fmaf(x * x, x - 1.2f, 1.0f / 3.0f);
-      ds = ce * fmaf(3.0f, x, -2.4f);
-    } else {
-      float xi = 1.0f / x;
-      float xi3 = xi * xi * xi;
-      s3 = c * (fmaf(x * x, fmaf(-1.0f / 3.0f, x, 1.2f), fmaf(-1.5f, x, 2.0f / 3.0f)) - xi3 * (1.0f / 480.0f));
-      ds = ce * (fmaf(-1.0f, x, 2.4f) - 1.5f * xi + xi3 * xi * xi * (1.0f / 160.0f));
-    }
-  } else {  // Plummer
-    float p = rsqrt_approx(r2 + f.eps2_f);
-    s3 = p * p * p;
-    ds = -3.0f * s3 * p * p;
-  }
-  if (VJP) {
-    float hd = sc.hd_f[kHTermsF - 1];
-#pragma unroll
-    for (int k = kHTermsF - 2; k >= 0; --k) hd = fmaf(hd, u2, sc.hd_f[k]);
-    // d/dr [h(u)/(2x_s)^3] / r = h'(u)/u / (2x_s)^5
-    D = ds - hd * f.hscale_f * f.inv2xs_f * f.inv2xs_f;
-  }
-  return s3 - h * f.hscale_f;
 }
 
 // Softened branch for two pairs at once (forward only): both B-spline pieces are

@@ -332,16 +332,6 @@ void launch_radix_scatter(int nblocks, cudaStream_t s, const int* keys_in, const
                                                                        hist, nblocks, nullptr, 0, 0);
 }
 
-__global__ void k_gather_pos(const double* __restrict__ src, const int* __restrict__ perm, int64_t n,
-                             double* __restrict__ dst) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  int64_t j = perm[k];
-  dst[k] = src[j];
-  dst[n + k] = src[n + j];
-  dst[2 * n + k] = src[2 * n + j];
-}
-
 // Gather the positions into walk order from the staged records and write the FP32 record of
 // each particle: its coordinates relative to the origin of its subtile and the id.
 __global__ void k_gather_pos_rel4(const double2* __restrict__ rec, const int* __restrict__ perm,
