@@ -1275,7 +1275,6 @@ static TraversalArgs base_args(p3m_sr_ctx* ctx) {
   a.n = ctx->n;
   a.rel4 = ctx->rel4;
   a.rel_scale = 1.0f;
-  a.unit = 1.0;
   a.pairs = ctx->pair_count;
   a.drift_slots = ctx->drift_slots;
   a.n_drift = ctx->n_drift;
@@ -1726,7 +1725,6 @@ extern "C" p3m_status p3m_sr_forces_noalloc(const p3m_sr_params* params, void* c
   a.pos = spos;
   a.rel4 = rel4;
   a.rel_scale = 1.0f;
-  a.unit = 1.0;
   a.offsets = offsets;
   a.chunks = chunks;
   a.n_chunks = small + 0;

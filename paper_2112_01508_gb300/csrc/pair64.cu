@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kMaxWarps64 * kWarp, 1) k_pair64(const __grid_
   const int n_chunks = *a.n_chunks;
   const int nparts = a.part_acc ? parts_for(n_chunks, a.part_items, kMaxParts64) : 1;
   const int n_items = n_chunks * nparts;
-  const Reach rc = make_reach(a);
+  const Reach rc = make_reach<true>(a, p.len);
   // an FP32 distance is within ~1e-5 x_r of the exact one (a little more after long drifts)
   const float slack = 1e-6f * rc.delta;
   const float cut = sqrtf(p.cut2) + slack, nearr = sqrtf(p.near2) + slack;
@@ -615,7 +615,6 @@ static cudaError_t launch_pair64_soft(p3m_sr_ctx* ctx, TraversalArgs a) {
   cudaError_t e = cudaFuncSetAttribute(k_pair64<VJP, SOFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxShared);
   if (e != cudaSuccess) return e;
   const int slot = VJP ? 1 : 0;
-  a.unit = p.len;
   a.rel_scale = rel_unit(ctx->prm.box) == 1.0 ? (float)p.len : 1.0f;
   for (int d = 0; d < 3; ++d) a.g.side32[d] = (float)(a.g.side64[d] * p.len);
   a.f.margin2_f = (float)(p.len * p.len * (ctx->prm.x_r * ctx->prm.x_r * (1.0 + 1e-4)));

@@ -18,7 +18,6 @@ struct TraversalArgs {
   const double* pos;          // FP64 path positions
   const float4* rel4;         // FP32 coordinates relative to the subtile, and its id
   float rel_scale;            // power of two that brings rel4 into the units of g.side32 and f.margin2_f
-  double unit;                // the same for lengths
   const int* offsets;         // S + 1 subtile offsets
   const Chunk* chunks;
   float4* part_acc;           // per (work item, lane) partial sums when chunks are split, or nullptr
@@ -81,14 +80,16 @@ struct WarpListOf {
 // subtile box and the receivers' box.  After drifts of total length delta since
 // the sort, a particle may lie up to delta outside the subtile it was sorted into:
 // the gap bound grows to x_r + delta and the block to x_r + 2 delta (receivers and
-// suppliers both moved).
+// suppliers both moved).  F64: in the unit `unit64` of the box, whatever scales the records; a bound that
+// has saturated is an error there (in FP32 no box is that large).
 struct Reach {
   int R[3];
   float sub2;   // squared gap bound
   float delta;  // total drift bound
 };
 
-__device__ __forceinline__ Reach make_reach(const TraversalArgs& a) {
+template <bool F64 = false>
+__device__ __forceinline__ Reach make_reach(const TraversalArgs& a, double unit64 = 1.0) {
   Reach r;
   float delta = 0.0f;
   for (int k = 0; k < a.n_drift; ++k) delta += a.drift_slots[k];
@@ -99,17 +100,21 @@ __device__ __forceinline__ Reach make_reach(const TraversalArgs& a) {
     r.delta = 0.0f;
     return r;
   }
-  r.delta = (float)(delta * a.unit);
-  const double dl = (double)delta * (1.0 + 1e-5) * a.unit;  // the float sum may round down
+  const auto unit = [&] {
+    if constexpr (F64) return unit64;
+    else return a.rel_scale;
+  }();
+  r.delta = (float)(delta * unit);
+  const double dl = (double)delta * (1.0 + 1e-5) * unit;  // the float sum may round down
   const double reach = sqrt((double)a.f.margin2_f) + dl;
-  const double half = 0.5 * a.g.box * a.unit;
-  if (!(reach + dl < half) || delta >= 3.0e38f) {  // (the bound of a drift saturates there)
+  const double half = 0.5 * a.g.box * unit;
+  if (!(reach + dl < half) || (F64 && delta >= 3.0e38f)) {  // (disp_bound saturates there)
     if ((threadIdx.x & 31) == 0 && a.err) atomicOr(a.err, kErrDrift);
   }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const double rr = fmin(reach + dl, half);
-    r.R[d] = (int)ceil(rr / (a.g.side64[d] * a.unit) * (1.0 + 1e-12));
+    r.R[d] = (int)ceil(rr / (a.g.side64[d] * unit) * (1.0 + 1e-12));
   }
   r.sub2 = (float)(reach * reach * (1.0 + 1e-6));
   return r;
