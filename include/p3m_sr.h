@@ -352,8 +352,9 @@ p3m_status p3m_sr_rung_kick_drift(p3m_sr_ctx* ctx, void* mom, int mom_precision,
  * displacement, and build_pairs / forces / vjp widen the subtile reach by the
  * sum of the bounds since the sort (more candidates, same pairs).  After 64
  * such drifts the sort is dropped (P3M_ERR_STATE until the next p3m_sr_sort);
- * a total drift with x_r + 2 drift >= L/2 latches P3M_ERR_STATE in the next
- * traversal.  Drifting any other array does not touch the sort.
+ * a total drift with x_r + 2 drift >= L/2 (or beyond the float range of its
+ * bound) latches P3M_ERR_STATE in the next traversal.  Drifting any other array
+ * does not touch the sort.
  */
 p3m_status p3m_sr_drift(p3m_sr_ctx* ctx, double* pos, const void* mom, int mom_precision,
                         double factor);

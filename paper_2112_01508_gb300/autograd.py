@@ -22,7 +22,8 @@ from .shortrange import ShortRange
 
 
 def _source(t: torch.Tensor) -> torch.Tensor:
-    """t without its history, packed where its elements lie apart (the kernels need (3, n) arrays)."""
+    """t without its history, copied where it is not contiguous: elements that lie apart are packed
+    (the strides of a dense transposed array stay, and the kernels' wrappers refuse it)."""
     t = t.detach()
     return t if t.is_contiguous() else t.clone()
 

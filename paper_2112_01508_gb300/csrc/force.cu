@@ -585,8 +585,9 @@ __global__ void k_parts_finish(TraversalArgs a) {
 // Bound: issue slots and the FP32 pipe (0.385 of the evaluated slots interact).  The
 // rotation's fixed cost, 6 shuffles, 2 shared loads and the loop, is paid per step, so a
 // step carries four (receiver, supplier) slots per lane instead of two: at 128^3 (654 M
-// ordered pairs) the forward takes 1.28 instead of 1.36 ms (1.07 instead of 1.22 G warp
-// instructions, the FP32 pipe 60% busy), the adjoint 1.82 instead of 1.96 ms.
+// ordered pairs) the forward took 1.28 instead of 1.36 ms and the adjoint 1.82 instead of
+// 1.96, and with the tile columns before the chunk's own cut off 1.25 and 1.79 ms (1.05 G
+// warp instructions instead of 1.22, the FP32 pipe 60% busy).
 // ---------------------------------------------------------------------------
 
 constexpr float kSymPad = 1e10f;  // padding supplier at -1e10, invalid receiver at +1e10: finite B, no hit
@@ -606,8 +607,8 @@ struct SymVjpSmem : SymSmem {
   float2 vz[kWarp];
 };
 
-// Resident blocks of 4 warps per SM: 5 for the forward (96 registers; 6 with spills and 7
-// within 0.5% of it at 128^3), 4 for the adjoint (122 registers; 5: 1% slower).
+// Resident blocks of 4 warps per SM: 5 for the forward (94 to 96 registers; 4 or 6 are 1-2%
+// slower at 128^3), 4 for the adjoint (122 to 128 registers; 5: 1% slower).
 constexpr int kSymMinBlocks = 5;
 constexpr int kSymVjpMinBlocks = 4;
 // Chunks are split into parts (slices of equal supplier counts) up to about three work items

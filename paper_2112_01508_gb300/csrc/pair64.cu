@@ -24,8 +24,10 @@
 // (27 G pairs/s; the FP64 pipe 87% busy, 97% of its lanes on interacting pairs, 17.8 lane
 // operations a pair), adjoint 5.6 ms; 9261 particles, 2.9 M pairs, Plummer: 0.19 and
 // 0.35 ms (0.45 and 0.80 with chunks split by subtiles instead of equal supplier counts).
-// Against 113-bit sums the force error fell from 6.7e-16 to 2.3e-16 (B-spline, relative
-// RMS), the adjoint's from 1.6e-15 to 4.3e-16.
+// Against 113-bit sums (relative RMS) the force error fell from 6.7e-16 to 2.3e-16 and the
+// adjoint's from 1.6e-15 to 4.3e-16 (B-spline), from 5.8e-16 to 1.8e-16 and from 6.8e-16 to
+// 3.3e-16 (Plummer).  A double evaluation of the closed forms shares the earlier kernel's
+// rounding and stands further from this one than from that: it is no measure below 1e-15.
 #include <algorithm>
 #include <cmath>
 
@@ -151,8 +153,11 @@ __device__ __noinline__ double2 bracket_direct(double r2, const ForceConsts& f, 
   return make_double2(B, D);
 }
 
-// B-spline softened form, r < r_sw = eps_B (Section 2.1.1): shape minus h, with
-// 1/r from a reciprocal square root refined to double precision.
+// B-spline softened form, r < r_sw = eps_B (Section 2.1.1): shape minus h.  1/r: with a first
+// value y and e = 1 - r^2 y^2, 1/r = y (1 - e)^(-1/2) = y (1 + e/2 + 3/8 e^2 + ...), the
+// binomial series cut after e^2 (one third-order Householder step).  y, from the truncated FP32
+// r^2 (2^-23) and the approximate root (2^-22.9), has |e| < 2^-21.3, so the rest of the series,
+// 5/16 e^3, is below 2^-65 and what remains is the rounding of the step itself.
 template <bool VJP>
 __device__ __forceinline__ bool soft_bspline(const Pair64Args& p, const Tables& T, double r2, float r2_f, float s_f,
                                              double& b, double& d) {
@@ -534,8 +539,8 @@ __global__ void k_parts_finish64(TraversalArgs a, double scale) {
   }
 }
 
-// The FP32 records are in the units of the positions where those fit a float with room for
-// a product with 2^-26, which is nearly always; else in units of the box's binary exponent.
+// The FP32 records are in the units of the positions where floats hold the box and, as normal
+// numbers, 2^-26 of it: nearly always.  Else in units of the box's binary exponent.
 double rel_unit(double box) {
   const int k = std::ilogb(box);
   return k >= -100 && k <= 120 ? 1.0 : std::ldexp(1.0, -k);

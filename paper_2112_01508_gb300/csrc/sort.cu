@@ -77,9 +77,9 @@ __global__ void k_bin(const double* __restrict__ pos, int64_t n, Geometry g, int
 // first particles have a neighbour kStageTiles tiles away in walk order.  Sets whose arrays
 // fit half of L2 are not staged at all: there the sectors cost less than the copy (128^3,
 // nothing carried: 202 us unstaged, 217 staged).
-// Out-of-place sort in random order: 15.4 M particles with 12 carried bytes 2540 -> 1532 us,
-// with 45 4174 -> 3256 us; 128^3 with 12 265 -> 259 us, with 45 405 -> 371 us; in nearly
-// sorted order unchanged or faster (15.4 M, 45 bytes: 1058 -> 946 us, from the loads issued
+// Out-of-place sort in random order, by this step alone: 15.4 M particles with 12 carried bytes
+// 2540 -> 1505 us, with 45 4174 -> 3064 us; 128^3 with 12 265 -> 259 us, with 45 405 -> 371 us;
+// in nearly sorted order faster (15.4 M, 45 bytes: 1060 -> 948 us, from the loads issued
 // together).
 constexpr int kStageTiles = 4;
 constexpr int64_t kStageBytes = 64 << 20;
@@ -197,8 +197,8 @@ __global__ void k_radix_hist(const int* __restrict__ keys, int64_t n, int shift,
 // issued before the rounds and the digits' output positions read once per block let 6 blocks
 // be resident (7 or 8 spill: 138 -> 160 us); ballots cost the same in every order, where
 // __match_any_sync took longer the more different digits a warp held.  Whole sorts before and
-// after: 15.4 M particles, nothing carried, nearly sorted 702 -> 649 us; 12 bytes carried,
-// nearly sorted 801 -> 751, in random order 1522 -> 1292; 128^3 in random order 250 -> 224.
+// after: 15.4 M particles, nothing carried, nearly sorted 702 -> 651 us; 12 bytes carried,
+// nearly sorted 801 -> 754, in random order 1522 -> 1268; 128^3 in random order 250 -> 224.
 constexpr int kScatterBlocks = 6;
 template <int STEPS>
 __global__ void __launch_bounds__(kRadixThreads, kScatterBlocks) k_radix_scatter(
@@ -398,7 +398,7 @@ struct WordGroup {
 // that the sectors of an array stay in L2 until its other particles have been read: 128^3 in
 // random order with 45 carried bytes moved 694 MB from DRAM in one pass (27% L2 hits).
 // Sort of 2.1 M in random order with 45 bytes 371 -> 334 us (404 before either), of 4.1 M
-// 977 -> 582 us with both; nearly sorted 246 -> 236 and 387 -> 357 us.  PHASED is a parameter, and
+// 916 -> 582 us; nearly sorted 246 -> 236 and 387 -> 357 us.  PHASED is a parameter, and
 // the two cases have code of their own, because counts that are not uniform constants cost a
 // nearly sorted input 10%.  Without carried arrays the kernel is the lighter one.
 constexpr int kPhase8 = 2, kPhase4 = 4;

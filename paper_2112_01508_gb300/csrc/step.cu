@@ -262,7 +262,9 @@ __global__ void __launch_bounds__(256, kKdMinBlocks) k_kick_drift(double* __rest
 
 // One kick of the rung-based leapfrog with the rung update (see p3m_sr_rung_kick) for
 // particle i.
-// (q: its momentum, in and out; written back if kicked)
+// (q: its momentum, in and out; written back if kicked.  Where nothing follows the kick the
+// compiler puts its load behind the rung test: 30 M particles of which none is due take 61.6 us
+// with momenta of either precision, as before q was passed in.)
 template <class M, class A>
 __device__ __forceinline__ void rung_kick_one(M* __restrict__ mom, M (&q)[3], const A* __restrict__ acc,
                                               int8_t* __restrict__ rung, int8_t* __restrict__ state, int64_t n,

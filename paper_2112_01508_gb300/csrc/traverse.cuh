@@ -80,8 +80,8 @@ struct WarpListOf {
 // subtile box and the receivers' box.  After drifts of total length delta since
 // the sort, a particle may lie up to delta outside the subtile it was sorted into:
 // the gap bound grows to x_r + delta and the block to x_r + 2 delta (receivers and
-// suppliers both moved).  F64: in the unit `unit64` of the box, whatever scales the records; a bound that
-// has saturated is an error there (in FP32 no box is that large).
+// suppliers both moved).  F64: lengths are multiplied by unit64, whatever the records' scale,
+// and a saturated bound is an error (in FP32 no box is that large).
 struct Reach {
   int R[3];
   float sub2;   // squared gap bound
